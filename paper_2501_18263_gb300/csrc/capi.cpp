@@ -248,7 +248,10 @@ dmrg_status dmrg_davidson(dmrg_handle* h, int32_t bond, double* psi, double tol,
     dmrg_status s = ensure_bond(h, bond);
     if (s != DMRG_OK) return s;
     int it = 0;
-    double e = h->eng->davidson(psi, tol, max_iter > 0 ? max_iter : 100, 24, &it, 1);
+    // an FP64 handle's iteration is followed with plain multiply-adds: bounded solves
+    // from far start vectors amplify a difference of one rounding without limit
+    double e = h->eng->davidson(psi, tol, max_iter > 0 ? max_iter : 100, 24, &it, 1,
+                                h->eng->problem().precision == DMRG_PREC_FP64);
     h->eng->exec()->sync();
     if (energy) *energy = e;
     if (iterations) *iterations = it;

@@ -788,7 +788,7 @@ void Engine::enlarge(bool left, const Block& blk, int site, Enlarged& E, OpSet& 
 // ---------------------------------------------------------------------------
 // renormalisation: new = U^T O U, fine-block by fine-block
 
-void Engine::renormalize(bool left, const Enlarged& E, const OpSet& eops, const Iso& iso, Block& out) {
+void Engine::renormalize(bool left, const Enlarged& E, const OpSet& eops, const Iso& iso, Block& out, bool plain) {
   (void)left;
   free_opset(out.ops);
   out.sec = iso.out;
@@ -814,8 +814,8 @@ void Engine::renormalize(bool left, const Enlarged& E, const OpSet& eops, const 
   std::vector<GemmSeg> s1, s2;
   int64_t used = 0;
   auto flush = [&]() {
-    if (!p1.empty()) ex_->gemm(p1, s1);
-    if (!p2.empty()) ex_->gemm(p2, s2);
+    if (!p1.empty()) ex_->gemm(p1, s1, plain);
+    if (!p2.empty()) ex_->gemm(p2, s2, plain);
     p1.clear(); p2.clear(); s1.clear(); s2.clear();
     used = 0;
   };

@@ -225,8 +225,10 @@ class Engine {
   // whether B_n / C_m exists or can be built from the isometries held (loaded or swept)
   bool left_buildable(int n) const;
   bool right_buildable(int m) const;
-  void build_left_blocks(int upto);     // B_0 .. B_upto from the loaded left isometries
-  void build_right_blocks(int downto);  // C_L .. C_downto
+  // B_0 .. B_upto and C_L .. C_downto from the loaded isometries.  plain: with plain
+  // FP64 multiply-adds (the operators of a basis the caller prepares; see Exec::gemm)
+  void build_left_blocks(int upto, bool plain = true);
+  void build_right_blocks(int downto, bool plain = true);
 
   // bond workspace
   void prepare_bond(int bond);
@@ -235,8 +237,9 @@ class Engine {
   int64_t psi_size() const { return psi_n_; }
   const BondStats& stats() const { return st_; }
 
-  void sigma(const double* psi, double* sig);                 // device pointers, FP64 path
-  void sigma_body(int precision);   // kernels of one sigma, psi_in_ -> sig_out_
+  void sigma(const double* psi, double* sig, bool plain = false);   // device pointers, FP64 path
+  void sigma_body(int precision);   // kernels of one sigma, psi_in_ -> sig_out_ (kPlain: FP64 multiply-adds)
+  static constexpr int kPlain = 2;
   // the same, from the bond's captured graph when possible (captured on first use
   // unless allow_capture is false: capturing instantiates a graph)
   void sigma_run(int precision, bool allow_capture = true);
@@ -252,7 +255,7 @@ class Engine {
   // refine = 1, after an FP64 refinement), 1 stopped at the residual floor of the
   // split-BF16 sigma (refine = 0 only), 2 max_iter reached, 3 no new direction
   // (the subspace is invariant).
-  double davidson(double* psi, double tol, int max_iter, int max_sub, int* iters_out, int refine);
+  double davidson(double* psi, double tol, int max_iter, int max_sub, int* iters_out, int refine, bool plain = false);
 
   // sweeps.  flags bit 0: FP64 refinement at every step of a split-BF16 sweep
   // (otherwise only at the step whose energy is reported); bit 1: mode
@@ -389,7 +392,7 @@ class Engine {
   int nparts_ = 1;
   // one captured CUDA graph per prepared bond and precision for the sigma steps of
   // Davidson (psi copied into psi_in_, result read from sig_out_ around the replay)
-  int graph_[2] = {-1, -1};
+  int graph_[3] = {-1, -1, -1};
   int64_t graph_runs_ = 0;
   void free_mixed();
   // sweep state
@@ -399,7 +402,7 @@ class Engine {
   void free_opset(OpSet& s);
   void alloc_opset(OpSet& s);
   void enlarge(bool left, const Block& blk, int site, Enlarged& E, OpSet& out);
-  void renormalize(bool left, const Enlarged& E, const OpSet& eops, const Iso& iso, Block& out);
+  void renormalize(bool left, const Enlarged& E, const OpSet& eops, const Iso& iso, Block& out, bool plain);
   void build_sigma_plan();
   std::vector<SigmaTerm> sigma_terms(bool keep_empty = false) const;   // terms of the prepared bond (all but H_L' (x) 1)
   void sigma_adjoint(const double* lam, const double* psi, const std::map<OpKey, std::map<std::pair<int, int>, int64_t>>& tl,

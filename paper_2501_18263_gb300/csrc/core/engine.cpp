@@ -130,26 +130,26 @@ bool Engine::right_buildable(int m) const {
   return false;
 }
 
-void Engine::build_left_blocks(int upto) {
+void Engine::build_left_blocks(int upto, bool plain) {
   for (int n = 0; n < upto; ++n) {
     if (lb_[n + 1].valid) continue;
     if (!liso_[n].valid) throw std::runtime_error("build_left_blocks: missing isometry");
     Enlarged E;
     OpSet eops;
     enlarge(true, lb_[n], n, E, eops);
-    renormalize(true, E, eops, liso_[n], lb_[n + 1]);
+    renormalize(true, E, eops, liso_[n], lb_[n + 1], plain);
     free_opset(eops);
   }
 }
 
-void Engine::build_right_blocks(int downto) {
+void Engine::build_right_blocks(int downto, bool plain) {
   for (int m = P_.L - 1; m >= downto; --m) {
     if (rb_[m].valid) continue;
     if (!riso_[m].valid) throw std::runtime_error("build_right_blocks: missing isometry");
     Enlarged E;
     OpSet eops;
     enlarge(false, rb_[m + 1], m, E, eops);
-    renormalize(false, E, eops, riso_[m], rb_[m]);
+    renormalize(false, E, eops, riso_[m], rb_[m], plain);
     free_opset(eops);
   }
 }
@@ -157,7 +157,7 @@ void Engine::build_right_blocks(int downto) {
 // ---------------------------------------------------------------------------
 // Davidson (FP64 subspace, Gram-Schmidt twice, Rayleigh-Ritz on the device)
 
-double Engine::davidson(double* psi, double tol, int max_iter, int max_sub, int* iters_out, int refine) {
+double Engine::davidson(double* psi, double tol, int max_iter, int max_sub, int* iters_out, int refine, bool plain) {
   if (bond_ < 0) throw std::runtime_error("davidson: no bond prepared");
   const int64_t n = psi_n_;
   max_sub = std::max(3, std::min(max_sub, 32));
@@ -184,7 +184,7 @@ double Engine::davidson(double* psi, double tol, int max_iter, int max_sub, int*
   const int prec = P_.precision;
 
   auto apply = [&](const double* in, double* out, int pr) {
-    if (pr == 0) sigma(in, out);
+    if (pr == 0) sigma(in, out, plain);
     else sigma_precision(in, out, pr);
   };
 
@@ -571,9 +571,9 @@ void Engine::truncate_and_move(bool ltr, int D, double* trunc_w, std::vector<int
   Enlarged Eold = E;
   tick(2);
   if (ltr) {
-    renormalize(true, EL_, EopsL_, iso, lb_[b + 1]);
+    renormalize(true, EL_, EopsL_, iso, lb_[b + 1], false);
   } else {
-    renormalize(false, ER_, EopsR_, iso, rb_[b + 1]);
+    renormalize(false, ER_, EopsR_, iso, rb_[b + 1], false);
   }
   tick(3);
   Enlarged ELold = EL_, ERold = ER_;
@@ -759,7 +759,7 @@ void Engine::init_sweep_state() {
     for (auto& M : mats) mp.push_back(M.data());
     load_right(m, out, mp);
   }
-  build_right_blocks(2);
+  build_right_blocks(2, false);
   prepare_bond(0);
   // random start vector
   if (psi_cur_) ex_->release(psi_cur_);
@@ -785,7 +785,7 @@ std::vector<double> Engine::run_sweeps(int nsw, const int* Dsched, double tol, i
     // a loaded or swept basis (e.g. after new integrals) is rebuilt at bond 0; the
     // swept wave function is kept when its layout still fits
     if (right_buildable(2)) {
-      build_right_blocks(2);
+      build_right_blocks(2, false);
       prepare_bond(0);
     }
     if (!(psi_cur_ && bond_ == 0 && psi_cur_cap_ == psi_n_)) init_sweep_state();

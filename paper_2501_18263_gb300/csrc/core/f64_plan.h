@@ -1,0 +1,76 @@
+// Work list of the tensor-core FP64 grouped GEMM (f64_tc.cu), built on the host from
+// the problems and segments of Exec::gemm_plan.
+//
+// Row side and column side.  A tile has up to 128 rows (the tensor core's lanes) and
+// up to 64 columns.  Problems of one launch that multiply by the same column side --
+// the same list of B operands, e.g. the same psi block for every operator's rows --
+// are stacked into one tall group so that their short rows fill the lanes; problems
+// that share their A list are stacked the same way with the two sides exchanged
+// (C^T = B^T A^T).  Every problem takes the orientation that needs fewer lanes.
+//
+// K runs over all segments of a problem, in octets (8 consecutive k of one segment,
+// the last of a segment padded with zeros).  A chunk is at most 24 octets: up to 192 k
+// the digit sums of the weights that matter are exact in the tensor core's FP32
+// accumulators.  Long sums are split over units (ranges of whole chunks), whose
+// partial sums are added in a fixed order by a second kernel.
+#pragma once
+#include <cstdint>
+#include <vector>
+
+#include "../exec.h"
+
+namespace dmrg {
+
+constexpr int F64_TM = 128;          // rows of a tile
+constexpr int F64_TN = 64;           // most columns of a tile
+constexpr int F64_CHUNK = 24;        // octets of a chunk
+constexpr int F64_PR = 8, F64_PC = 4;   // rows and columns of a piece
+
+// operand of one segment, seen from its side: element (r, k) at p[r ld + k] (kt even)
+// or p[k ld + r] (kt odd); K = kt / 2
+struct F64Ref {
+  const double* p;
+  int ld, kt;
+};
+// one problem at its place in a group: rows [pre, pre + m2 / 2) of the stack, the
+// operands of its segments at s0, accumulate flag in bit 0 of m2
+struct F64Row {
+  double* C;
+  double alpha;
+  int ldc, s0, pre, m2;
+};
+// one unit: a tile (stack rows row0 .., columns n0 ..) and a range of noct octets that
+// begins at k0 of segment sg; part >= 0: the unit's sum goes to that place of the
+// partial sums (column-major, 128 rows), otherwise to C
+struct F64Unit {
+  int pos0, npos;    // problems the tile's rows belong to
+  int row0, rows, n0, nt;
+  int cs, nseg;      // column operands: refs cs .. cs + nseg - 1
+  int sg, k0, noct;
+  int trans;         // 1: sides exchanged, C(row, col) at C[row + col ldc]
+  int64_t part;
+};
+struct F64Red {
+  int pos0, row0, rows, n0, nt, trans, nparts, n16;
+  int64_t part;
+};
+
+struct F64PlanHost {
+  std::vector<F64Ref> rowref, colref;
+  std::vector<F64Row> rows;
+  std::vector<F64Unit> units;
+  // the tiles unsplit, longest sum first, and the prefix sums of their 8 x 4 pieces
+  // (the plain FP64 kernel: one warp per piece)
+  std::vector<F64Unit> tiles;
+  std::vector<int> pieces;
+  std::vector<F64Red> reds;
+  int64_t npart = 0;   // doubles of the partial sums
+};
+
+// what: F64_UNITS the tensor-core form, F64_TILES the plain one (alone, its problems
+// are not stacked), or both
+enum { F64_UNITS = 1, F64_TILES = 2 };
+F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int nsm,
+                           int what = F64_UNITS | F64_TILES);
+
+}  // namespace dmrg

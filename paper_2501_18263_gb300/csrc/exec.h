@@ -143,11 +143,14 @@ class Exec {
 
   // grouped element-wise Kronecker accumulation (operator blocking)
   virtual void kron(const std::vector<KronGroup>& g, const std::vector<KronTask>& t) = 0;
-  // grouped, segmented FP64 GEMM (one-shot upload)
-  virtual void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) = 0;
+  // grouped, segmented FP64 GEMM (one-shot upload).  plain: every element by FP64
+  // multiply-adds in the order of its segments and k, so that its rounding does not
+  // depend on the launch; otherwise the executor may use its tensor-core form (error
+  // no larger, another rounding sequence)
+  virtual void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain = false) = 0;
   // persistent plans (uploaded once, replayed during Davidson)
   virtual int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) = 0;
-  virtual void gemm_run(int plan) = 0;
+  virtual void gemm_run(int plan, bool plain = false) = 0;
   virtual void plan_free(int plan) = 0;
   virtual void diag(const std::vector<DiagTask>& t) = 0;
   // generalised Fock matrix F_pq = sum_r t_pr g1_qr + sum_rst v_prst g2_qrst and the

@@ -1,5 +1,5 @@
 // CUDA executor: the sm_103a kernels behind the host core's numerical steps.
-//   gemm_f64      grouped, segmented FP64 GEMM (the FP64 sigma / Ren / StVec path)
+//   gemm          grouped, segmented FP64 GEMM (f64_tc.cu: the FP64 sigma / Ren / StVec path)
 //   kron          grouped Kronecker accumulation (operator blocking)
 //   mdot/lincomb  Davidson Gram-Schmidt and Ritz vectors (deterministic reductions)
 //   ritz          cyclic Jacobi eigensolver of the small Rayleigh-Ritz matrix
@@ -18,6 +18,7 @@
 
 #include "../exec.h"
 #include "../exec_errors.h"
+#include "f64_tc.h"
 #include "mixed.h"
 #include "tridiag_dc.h"
 
@@ -31,93 +32,6 @@ namespace dmrg {
       throw CudaError(std::string(#x) + ": " + cudaGetErrorString(e_));               \
     }                                                                                  \
   } while (0)
-
-// ---------------------------------------------------------------------------
-// grouped FP64 GEMM: one CTA per 64 x 64 output tile, K loop over all segments
-
-struct GemmTile {
-  int prob, m0, n0, pad;
-};
-
-constexpr int TM = 64, TN = 64, TK = 16;
-
-__global__ void __launch_bounds__(256) gemm_f64_kernel(const GemmTile* __restrict__ tiles,
-                                                       const GemmProb* __restrict__ probs,
-                                                       const GemmSeg* __restrict__ segs) {
-  __shared__ double As[TK][TM + 1];
-  __shared__ double Bs[TK][TN + 1];
-  const GemmTile tl = tiles[blockIdx.x];
-  const GemmProb p = probs[tl.prob];
-  const int tid = threadIdx.x;
-  // warp w owns rows 16 (w / 2) .. +15 and columns 32 (w % 2) .. +31 of the
-  // tile, its lanes 4 x 8 sub-tiles of 4 x 4; a warp whose rows or columns lie
-  // wholly past a ragged edge skips the multiply-adds (warp-uniform test)
-  const int warp = tid >> 5, lane = tid & 31;
-  const int ty = 4 * (warp >> 1) + (lane >> 3), tx = 8 * (warp & 1) + (lane & 7);
-  double acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  const int Mt = min(TM, p.M - tl.m0), Nt = min(TN, p.N - tl.n0);
-  const bool busy = 16 * (warp >> 1) < Mt && 32 * (warp & 1) < Nt;
-  for (int s = p.s0; s < p.s1; ++s) {
-    const GemmSeg g = segs[s];
-    for (int k0 = 0; k0 < g.K; k0 += TK) {
-      const int Kt = min(TK, g.K - k0);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = tid + 256 * r;
-        int m, k;
-        if (g.ta == 0) { m = i >> 4; k = i & 15; } else { m = i & 63; k = i >> 6; }
-        double a = 0.0;
-        if (m < Mt && k < Kt) {
-          const int64_t gm = tl.m0 + m, gk = k0 + k;
-          a = g.ta == 0 ? g.A[gm * g.lda + gk] : g.A[gk * g.lda + gm];
-        }
-        As[k][m] = a;
-        int n, kb;
-        if (g.tb == 0) { n = i & 63; kb = i >> 6; } else { n = i >> 4; kb = i & 15; }
-        double b = 0.0;
-        if (n < Nt && kb < Kt) {
-          const int64_t gn = tl.n0 + n, gk = k0 + kb;
-          b = g.tb == 0 ? g.B[gk * g.ldb + gn] : g.B[gn * g.ldb + gk];
-        }
-        Bs[kb][n] = b;
-      }
-      __syncthreads();
-      if (busy) {
-        // a ragged K step (Kt < TK: the last one of a segment) runs only its own k
-#pragma unroll 4
-        for (int k = 0; k < Kt; ++k) {
-          double a[4], b[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a[i] = As[k][ty * 4 + i];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx * 4 + j];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-      }
-      __syncthreads();
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = ty * 4 + i;
-    if (m >= Mt) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = tx * 4 + j;
-      if (n >= Nt) continue;
-      double* c = p.C + int64_t(tl.m0 + m) * p.ldc + tl.n0 + n;
-      const double v = p.alpha * acc[i][j];
-      *c = p.accumulate ? *c + v : v;
-    }
-  }
-}
 
 // ---------------------------------------------------------------------------
 // grouped Kronecker accumulation
@@ -861,23 +775,54 @@ class CudaExec : public Exec {
   }
 
   struct Plan {
-    GemmTile* tiles = nullptr;
-    GemmProb* probs = nullptr;
-    GemmSeg* segs = nullptr;
-    int ntiles = 0;
+    void* mem = nullptr;   // one allocation: every table of the plan
+    F64Unit* units = nullptr;
+    F64Row* rows = nullptr;
+    F64Ref* rowref = nullptr;
+    F64Ref* colref = nullptr;
+    F64Red* reds = nullptr;
+    F64Unit* tiles = nullptr;
+    int* pieces = nullptr;
+    int* next = nullptr;
+    double* part = nullptr;
+    int nunits = 0, nreds = 0, ntiles = 0, npieces = 0;
     bool live = false;
   };
 
   int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) override {
+    return f64_plan(p, s, F64_UNITS | F64_TILES);
+  }
+  int f64_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int what) {
+    const F64PlanHost h = f64_build_plan(p, s, nsm_, what);
     Plan pl;
-    std::vector<GemmTile> tiles;
-    for (size_t i = 0; i < p.size(); ++i)
-      for (int m0 = 0; m0 < p[i].M; m0 += TM)
-        for (int n0 = 0; n0 < p[i].N; n0 += TN) tiles.push_back(GemmTile{int(i), m0, n0, 0});
-    pl.ntiles = int(tiles.size());
-    pl.tiles = upload(tiles);
-    pl.probs = upload(p);
-    pl.segs = upload(s);
+    pl.nunits = int(h.units.size());
+    pl.nreds = int(h.reds.size());
+    pl.ntiles = int(h.tiles.size());
+    pl.npieces = h.pieces.empty() ? 0 : h.pieces.back();
+    // tables side by side, each at a multiple of 16 bytes; the two claim counters first
+    std::vector<char> buf(16, 0);
+    auto place = [&](const auto& v) {
+      const size_t at = buf.size(), n = v.size() * sizeof(v[0]);
+      buf.resize(at + ((n + 15) & ~size_t(15)));
+      if (n) std::memcpy(buf.data() + at, v.data(), n);
+      return at;
+    };
+    buf.reserve(16 * 8 + sizeof(F64Unit) * (h.units.size() + h.tiles.size()) + sizeof(F64Row) * h.rows.size() +
+                sizeof(F64Ref) * (h.rowref.size() + h.colref.size()) + sizeof(F64Red) * h.reds.size() +
+                sizeof(int) * h.pieces.size());
+    const size_t o0 = place(h.units), o1 = place(h.rows), o2 = place(h.rowref), o3 = place(h.colref),
+                 o4 = place(h.reds), o5 = place(h.tiles), o6 = place(h.pieces);
+    char* d = reinterpret_cast<char*>(upload(buf));
+    pl.mem = d;
+    pl.next = reinterpret_cast<int*>(d);
+    pl.units = reinterpret_cast<F64Unit*>(d + o0);
+    pl.rows = reinterpret_cast<F64Row*>(d + o1);
+    pl.rowref = reinterpret_cast<F64Ref*>(d + o2);
+    pl.colref = reinterpret_cast<F64Ref*>(d + o3);
+    pl.reds = reinterpret_cast<F64Red*>(d + o4);
+    pl.tiles = reinterpret_cast<F64Unit*>(d + o5);
+    pl.pieces = reinterpret_cast<int*>(d + o6);
+    if (h.npart) pl.part = static_cast<double*>(alloc(sizeof(double) * size_t(h.npart)));
     pl.live = true;
     for (size_t i = 0; i < plans_.size(); ++i)
       if (!plans_[i].live) {
@@ -887,23 +832,29 @@ class CudaExec : public Exec {
     plans_.push_back(pl);
     return int(plans_.size() - 1);
   }
-  void gemm_run(int id) override {
+  void gemm_run(int id, bool plain) override {
     Plan& pl = plans_.at(id);
-    if (!pl.ntiles) return;
-    launch(PROF_GEMM, [&] { gemm_f64_kernel<<<pl.ntiles, 256, 0, st_>>>(pl.tiles, pl.probs, pl.segs); });
+    if (!(plain ? pl.ntiles : pl.nunits)) return;
+    launch(PROF_GEMM, [&] {
+      if (plain) {
+        launch_gemm_f64_plain(pl.tiles, pl.pieces, pl.ntiles, pl.npieces, pl.rows, pl.rowref, pl.colref, st_);
+        return;
+      }
+      launch_gemm_f64_tc(pl.units, pl.nunits, pl.rows, pl.rowref, pl.colref, pl.part, pl.reds, pl.nreds, pl.next, err_, nsm_,
+                         st_);
+    });
   }
   void free_plan_mem(Plan& p) {
     if (!p.live) return;
-    cudaFreeAsync(p.tiles, st_);
-    cudaFreeAsync(p.probs, st_);
-    cudaFreeAsync(p.segs, st_);
+    cudaFreeAsync(p.mem, st_);
+    if (p.part) cudaFreeAsync(p.part, st_);
     p.live = false;
   }
   void plan_free(int id) override { free_plan_mem(plans_.at(id)); }
-  void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) override {
+  void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain) override {
     if (p.empty()) return;
-    int id = gemm_plan(p, s);
-    gemm_run(id);
+    int id = f64_plan(p, s, plain ? F64_TILES : F64_UNITS);
+    gemm_run(id, plain);
     plan_free(id);
   }
   void orbital_gradient(int L, const double* t, const double* v, const double* g1, const double* g2,
@@ -1362,7 +1313,7 @@ class CudaExec : public Exec {
         q.s1 = int(S.size());
         P.push_back(q);
       }
-      gemm(P, S);
+      gemm(P, S, false);
     }
     // 5. order
     launch(PROF_EIG, [&] { syev_sort_kernel<<<unsigned((ncol + 255) / 256), 256, 0, st_>>>(dj, dpn, nj); });
