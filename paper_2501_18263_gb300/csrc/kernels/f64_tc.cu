@@ -99,6 +99,22 @@ __device__ __forceinline__ uint32_t f64_idesc(int n) {
   return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(F64_TM >> 4) << 24);
 }
 
+// the MMAs of one 16-k stage of an N-column tile: digit i of A with digits j .. of B, as
+// many as fit N = 256, into the accumulators i + j ..; every operand a constant away
+// from the stage's descriptors (computing them per MMA took ten times the MMAs' time)
+template <int N>
+__device__ __forceinline__ void stage_mmas(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+  constexpr int PER = 256 / N < F64_DIGITS ? 256 / N : F64_DIGITS;
+#pragma unroll
+  for (int i = 0; i < F64_DIGITS; ++i)
+#pragma unroll
+    for (int j = 0; j < F64_DIGITS - i; j += PER) {
+      const int nd = PER < F64_DIGITS - i - j ? PER : F64_DIGITS - i - j;
+      mma(d + uint32_t((i + j) * N), a + uint64_t(i * F64_TM * 2), b + uint64_t(j * N * 2), f64_idesc(nd * N),
+          i == 0 ? acc : 1u);
+    }
+}
+
 // TMEM 32 lanes x 4 columns of the eight accumulators (n columns apart) and the wait
 __device__ __forceinline__ void tmem_ld8x4(uint32_t t, uint32_t n, float (&v)[8][4]) {
   uint32_t a[32];
@@ -438,18 +454,17 @@ __global__ void __maxnreg__(REGS)
             ++used1;
           }
           const uint32_t d = tmem + 256u * b0;
-          const int per = 256 / n;   // digits of B per MMA
           for (int t = 0; t < (nOct + 1) >> 1; ++t, ++step) {
             const int st = step % STAGES;
             if (!mbar_wait(full(st), (step / STAGES) & 1, abort_flag, err, 15)) goto mma_done;
             fence_after();
-            const uint32_t a = saddr(smem + st * STAGE_BYTES), b = a + A_BYTES;
-            for (int i = 0; i < F64_DIGITS; ++i)
-              for (int j = 0; j < F64_DIGITS - i; j += per) {
-                const int nd = min(per, F64_DIGITS - i - j);
-                mma(d + uint32_t((i + j) * n), f64_sdesc(a + i * F64_TM * 32), f64_sdesc(b + j * n * 32),
-                    f64_idesc(nd * n), (t == 0 && i == 0) ? 0u : 1u);
-              }
+            const uint32_t base = saddr(smem + st * STAGE_BYTES);
+            const uint64_t da = f64_sdesc(base), db = f64_sdesc(base + A_BYTES);
+            const uint32_t acc = t > 0;
+            if (n == 16) stage_mmas<16>(d, da, db, acc);
+            else if (n == 32) stage_mmas<32>(d, da, db, acc);
+            else if (n == 48) stage_mmas<48>(d, da, db, acc);
+            else stage_mmas<64>(d, da, db, acc);
             mma_commit(empty(st));
           }
           mma_commit(acc_full(b0));

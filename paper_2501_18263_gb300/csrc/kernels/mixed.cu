@@ -101,6 +101,19 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 
+// the six products of one 16-k step: planes (hi, mid, lo) 512 bytes apart.  Every
+// operand is a constant away from the stage's descriptors, and a full tile's
+// instruction descriptor is a constant: an MMA whose operands are computed one by one
+// takes longer to issue (about 300 clocks) than to run (64)
+__device__ __forceinline__ void k16_mmas(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  mma(d, a, b, id, acc);
+  mma(d + 128, a, b + 32, id, acc);
+  mma(d + 128, a + 32, b, id, 1u);
+  mma(d + 128, a, b + 64, id, 1u);
+  mma(d + 128, a + 32, b + 32, id, 1u);
+  mma(d + 128, a + 64, b, id, 1u);
+}
+
 __device__ __forceinline__ uint16_t bf_bits(__nv_bfloat16 x) { return __bfloat16_as_ushort(x); }
 
 // error-free sum of two floats (TwoSum)
@@ -232,20 +245,16 @@ __global__ void __maxnreg__(96)
           dbase = tmem + 256u * b;
         }
         fence_after();
-        const uint32_t id = idesc(si.nmma);
         const uint32_t base = saddr(smem + st * STAGE_BYTES);
-        for (int kk = 0; kk < si.ksub; ++kk) {
-          const uint32_t o = kk * 256;
-          const uint64_t a0 = sdesc(base + o), a1 = sdesc(base + 512 + o), a2 = sdesc(base + 1024 + o);
-          const uint64_t b0 = sdesc(base + OPER_BYTES + o), b1 = sdesc(base + OPER_BYTES + 512 + o),
-                         b2 = sdesc(base + OPER_BYTES + 1024 + o);
-          const uint32_t acc = (in_chunk == 0 && kk == 0) ? 0u : 1u;
-          mma(dbase, a0, b0, id, acc);
-          mma(dbase + 128, a0, b1, id, acc);
-          mma(dbase + 128, a1, b0, id, 1u);
-          mma(dbase + 128, a0, b2, id, 1u);
-          mma(dbase + 128, a1, b1, id, 1u);
-          mma(dbase + 128, a2, b0, id, 1u);
+        const uint64_t da = sdesc(base), db = sdesc(base + OPER_BYTES);
+        const uint32_t acc = in_chunk != 0;
+        if (si.nmma == MIX_TN) {
+          k16_mmas(dbase, da, db, idesc(MIX_TN), acc);
+          if (si.ksub > 1) k16_mmas(dbase, da + 16, db + 16, idesc(MIX_TN), 1u);
+        } else {
+          const uint32_t id = idesc(si.nmma);
+          k16_mmas(dbase, da, db, id, acc);
+          if (si.ksub > 1) k16_mmas(dbase, da + 16, db + 16, id, 1u);
         }
         mma_commit(empty(st));
         if (++in_chunk == CHUNK || si.last) {
