@@ -35,29 +35,17 @@ namespace {
 
 using TargetMap = std::map<OpKey, std::map<std::pair<int, int>, int64_t>>;
 
-// one blocking step: its contributions and the fine blocks whose adjoints it reads
-struct AdjStep {
-  Enlarged E;
-  std::vector<BlockingTerm> bt;
-  TargetMap tgt;   // (operator, fine block) -> offset in the step's adjoint arena
-  int64_t n = 0;
-};
+TargetMap target_map(const AdjStep& s) {
+  TargetMap m;
+  for (const AdjTarget& t : s.tgt) m[s.keys[size_t(t.key)]][{t.rf, t.cf}] = t.off;
+  return m;
+}
 
-}  // namespace
-
-namespace {
-
-AdjStep make_step(const Engine& eng, bool left, const Block& blk, int site) {
-  AdjStep s;
-  s.bt = eng.blocking_terms(left, blk, site, s.E);
-  for (const BlockingTerm& x : s.bt) {
-    auto& m = s.tgt[x.key];
-    auto it = m.find({x.rf, x.cf});
-    if (it != m.end()) continue;
-    m[{x.rf, x.cf}] = s.n;
-    s.n += int64_t(s.E.f_dim[x.rf]) * s.E.f_dim[x.cf];
-  }
-  return s;
+// blocks of an operator set (ids 0 .. count - 1 in (operator, block) order)
+int block_count(const OpSet& s) {
+  int n = 0;
+  for (auto& kv : s.ops) n += int(kv.second.blk.size());
+  return n;
 }
 
 }  // namespace
@@ -85,63 +73,65 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
   raw.assign(size_t(L2 + L2 * L2), 0.0);
   if (!lb_[b].valid || !rb_[b + 2].valid) throw std::runtime_error("integral_gradient: blocks not built");
 
-  // Frobenius products of the adjoints with the operators they multiply, spread over
-  // the integrals of each coefficient (host, in a fixed order)
-  auto spread = [&](const std::vector<DotTask>& dt, const std::vector<const Lin*>& dl) {
-    if (dt.empty()) return;
-    double* d = static_cast<double*>(ex_->alloc(dt.size() * sizeof(double)));
-    ex_->dots(dt, d);
-    std::vector<double> h(dt.size());
-    ex_->d2h(h.data(), d, h.size() * sizeof(double));
-    ex_->release(d);
-    for (size_t i = 0; i < h.size(); ++i)
-      for (const auto& w : dl[i]->w) raw[size_t(w.first)] += w.second * h[i];
-  };
-
   // blocking step backwards: adjoint of the block operators (arena of blk.ops's
-  // layout, allocated here) and the coefficient derivatives
+  // layout, allocated here) and the coefficient derivatives: Frobenius products of the
+  // adjoints with the operators they multiply, spread over the integrals of each
+  // coefficient (host, in a fixed order)
   auto back_blocking = [&](const AdjStep& st, const Block& blk, const double* adjE) -> double* {
     const int64_t nb = std::max<int64_t>(blk.ops.n_elem, 1);
     double* ob = static_cast<double*>(ex_->alloc(size_t(nb) * sizeof(double)));
     ex_->zero(ob, size_t(nb) * sizeof(double));
-    std::map<std::pair<const Op*, int>, std::vector<KronTask>> groups;
+    // contributions dealt out to the source blocks (counting sort by block id, so that
+    // each block sums its own in list order), and the products with a coefficient
+    const int nblk = block_count(blk.ops);
+    std::vector<const OpBlk*> blks(static_cast<size_t>(nblk));
+    for (auto& kv : blk.ops.ops)
+      for (auto& b : kv.second.blk) blks[size_t(b.id)] = &b;
+    std::vector<int> first(size_t(nblk) + 1, 0);
+    size_t nd = 0;
+    for (const AdjTerm& x : st.terms) {
+      if (x.src && x.val != 0.0) ++first[size_t(x.src->blk[size_t(x.src_blk)].id) + 1];
+      nd += x.w1 > x.w0;
+    }
+    for (int i = 0; i < nblk; ++i) first[size_t(i) + 1] += first[size_t(i)];
+    std::vector<KronTask> kt(static_cast<size_t>(first[size_t(nblk)]));
     std::vector<DotTask> dt;
-    std::vector<const Lin*> dl;
-    for (const BlockingTerm& x : st.bt) {
-      const int64_t go = st.tgt.at(x.key).at({x.rf, x.cf});
-      const int rows = st.E.f_dim[x.rf], cols = st.E.f_dim[x.cf];
-      const double* g = adjE + go;
-      if (x.src) {
-        const double val = lin_value(x.coef);
-        if (val != 0.0) groups[{x.src, x.src_blk}].push_back(KronTask{g, cols, x.trans, val});
-      }
-      if (!x.coef.w.empty()) {
-        if (x.src) {
-          const OpBlk& sb = x.src->blk[x.src_blk];
-          dt.push_back(DotTask{g, blk.ops.arena + sb.off, cols, sb.cols, rows, cols, x.trans});
-        } else {
-          dt.push_back(DotTask{g, nullptr, cols, 0, rows, cols, 2});
+    std::vector<const AdjTerm*> dl;
+    dt.reserve(nd);
+    dl.reserve(nd);
+    {
+      std::vector<int> at(first.begin(), first.end() - 1);
+      for (const AdjTarget& tg : st.tgt) {
+        const int rows = st.E.f_dim[tg.rf], cols = st.E.f_dim[tg.cf];
+        const double* g = adjE + tg.off;
+        for (int k = tg.t0; k < tg.t1; ++k) {
+          const AdjTerm& x = st.terms[size_t(k)];
+          const OpBlk* sb = x.src ? &x.src->blk[size_t(x.src_blk)] : nullptr;
+          if (sb && x.val != 0.0) kt[size_t(at[size_t(sb->id)]++)] = KronTask{g, cols, x.trans, x.val};
+          if (x.w1 > x.w0) {
+            dt.push_back(sb ? DotTask{g, blk.ops.arena + sb->off, cols, sb->cols, rows, cols, x.trans}
+                            : DotTask{g, nullptr, cols, 0, rows, cols, 2});
+            dl.push_back(&x);
+          }
         }
-        dl.push_back(&x.coef);
       }
     }
     std::vector<KronGroup> kg;
-    std::vector<KronTask> kt;
-    for (auto& gv : groups) {
-      const OpBlk& sb = gv.first.first->blk[gv.first.second];
-      KronGroup g;
-      g.dst = ob + sb.off;
-      g.ld = sb.cols;
-      g.rows = sb.rows;
-      g.cols = sb.cols;
-      g.t0 = int(kt.size());
-      g.accumulate = 0;
-      kt.insert(kt.end(), gv.second.begin(), gv.second.end());
-      g.t1 = int(kt.size());
-      kg.push_back(g);
+    for (int i = 0; i < nblk; ++i) {
+      if (first[size_t(i)] == first[size_t(i) + 1]) continue;
+      const OpBlk& sb = *blks[size_t(i)];
+      kg.push_back(KronGroup{ob + sb.off, sb.cols, sb.rows, sb.cols, first[size_t(i)], first[size_t(i) + 1], 0});
     }
     if (!kg.empty()) ex_->kron(kg, kt);
-    spread(dt, dl);
+    if (!dt.empty()) {
+      double* d = static_cast<double*>(ex_->alloc(dt.size() * sizeof(double)));
+      ex_->dots(dt, d);
+      std::vector<double> h(dt.size());
+      ex_->d2h(h.data(), d, h.size() * sizeof(double));
+      ex_->release(d);
+      for (size_t i = 0; i < h.size(); ++i)
+        for (int k = dl[i]->w0; k < dl[i]->w1; ++k) raw[size_t(st.w[size_t(k)].first)] += st.w[size_t(k)].second * h[i];
+    }
     return ob;
   };
 
@@ -158,24 +148,43 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
       if (c < 0 || E.coarse.dim[c] != iso.rows[k]) throw std::runtime_error("adjoint: isometry and enlarged basis differ");
       c2s[c] = int(k);
     }
-    // W(op, block) = adj B'{r <- c} U_c^T (dr x rows_c), then adj E{fr, fc} = U_r{fr rows} W{fc cols}
-    struct Need { const Op* op; int bi; std::vector<std::pair<int64_t, std::pair<int, int>>> t; };
-    std::map<std::pair<const Op*, int>, Need> need;
-    for (auto& kv : nx.tgt) {
-      auto oit = B.ops.ops.find(kv.first);
-      if (oit == B.ops.ops.end()) continue;
-      const Op& bo = oit->second;
-      for (auto& tv : kv.second) {
-        const int rf = tv.first.first, cf = tv.first.second;
-        const int r = c2s[E.f_coarse[rf]], c = c2s[E.f_coarse[cf]];
-        if (r < 0 || c < 0) continue;
-        auto bit = bo.by_col.find(c);
-        if (bit == bo.by_col.end() || bo.blk[bit->second].r != r) continue;
-        Need& nd = need[{&bo, bit->second}];
-        nd.op = &bo;
-        nd.bi = bit->second;
-        nd.t.push_back({tv.second, {rf, cf}});
+    // W(op, block) = adj B'{r <- c} U_c^T (dr x rows_c), then adj E{fr, fc} = U_r{fr rows} W{fc cols}:
+    // the targets of every block operator's block, by block id
+    std::vector<const Op*> kop(nx.keys.size(), nullptr);
+    for (size_t k = 0; k < nx.keys.size(); ++k) {
+      auto it = B.ops.ops.find(nx.keys[k]);
+      if (it != B.ops.ops.end()) kop[k] = &it->second;
+    }
+    const int nblk = block_count(B.ops);
+    std::vector<const OpBlk*> blks(size_t(nblk), nullptr);
+    for (auto& kv : B.ops.ops)
+      for (auto& b : kv.second.blk) blks[size_t(b.id)] = &b;
+    // block of the operator at column sector c (one per column), -1 where it has none
+    std::vector<int> tblk(nx.tgt.size(), -1), first(size_t(nblk) + 1, 0);
+    {
+      int key = -1;
+      std::vector<int> bycol;
+      for (size_t i = 0; i < nx.tgt.size(); ++i) {
+        const AdjTarget& t = nx.tgt[i];
+        const Op* bo = kop[size_t(t.key)];
+        if (!bo) continue;
+        if (t.key != key) {
+          key = t.key;
+          bycol.assign(iso.out.q.size(), -1);
+          for (auto& b : bo->blk) bycol[size_t(b.c)] = b.id;
+        }
+        const int r = c2s[E.f_coarse[t.rf]], c = c2s[E.f_coarse[t.cf]];
+        if (r < 0 || c < 0 || bycol[size_t(c)] < 0 || blks[size_t(bycol[size_t(c)])]->r != r) continue;
+        tblk[i] = bycol[size_t(c)];
+        ++first[size_t(tblk[i]) + 1];
       }
+    }
+    for (int i = 0; i < nblk; ++i) first[size_t(i) + 1] += first[size_t(i)];
+    std::vector<int> order(static_cast<size_t>(first[size_t(nblk)]));
+    {
+      std::vector<int> at(first.begin(), first.end() - 1);
+      for (size_t i = 0; i < nx.tgt.size(); ++i)
+        if (tblk[i] >= 0) order[size_t(at[size_t(tblk[i])]++)] = int(i);
     }
     const int64_t cap = int64_t(1) << 27;
     double* W = nullptr;
@@ -189,9 +198,9 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
       p1.clear(); p2.clear(); s1.clear(); s2.clear();
       used = 0;
     };
-    for (auto& nv : need) {
-      const Need& nd = nv.second;
-      const OpBlk& bk = nd.op->blk[nd.bi];
+    for (int bi = 0; bi < nblk; ++bi) {
+      if (first[size_t(bi)] == first[size_t(bi) + 1]) continue;
+      const OpBlk& bk = *blks[size_t(bi)];
       const int r = bk.r, c = bk.c;
       const int dr = iso.out.dim[r], dc = iso.out.dim[c], rows_c = iso.rows[c];
       const int64_t sz = int64_t(dr) * rows_c;
@@ -216,10 +225,11 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
       s1.push_back(GemmSeg{ob + bk.off, iso.mat[c], dc, dc, dc, 0, 1});
       q.s1 = int(s1.size());
       p1.push_back(q);
-      for (auto& tg : nd.t) {
-        const int rf = tg.second.first, cf = tg.second.second;
+      for (int k = first[size_t(bi)]; k < first[size_t(bi) + 1]; ++k) {
+        const AdjTarget& tg = nx.tgt[size_t(order[size_t(k)])];
+        const int rf = tg.rf, cf = tg.cf;
         GemmProb q2;
-        q2.C = ge + tg.first;
+        q2.C = ge + tg.off;
         q2.ldc = E.f_dim[cf];
         q2.M = E.f_dim[rf];
         q2.N = E.f_dim[cf];
@@ -237,13 +247,13 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
   };
 
   // 1. the bond
-  AdjStep SL = make_step(*this, true, lb_[b], b);
-  AdjStep SR = make_step(*this, false, rb_[b + 2], b + 1);
+  AdjStep SL = adjoint_step(true, lb_[b], b);
+  AdjStep SR = adjoint_step(false, rb_[b + 2], b + 1);
   double* gl = static_cast<double*>(ex_->alloc(size_t(std::max<int64_t>(SL.n, 1)) * sizeof(double)));
   double* gr = static_cast<double*>(ex_->alloc(size_t(std::max<int64_t>(SR.n, 1)) * sizeof(double)));
   ex_->zero(gl, size_t(std::max<int64_t>(SL.n, 1)) * sizeof(double));
   ex_->zero(gr, size_t(std::max<int64_t>(SR.n, 1)) * sizeof(double));
-  sigma_adjoint(lam, psi, SL.tgt, gl, SR.tgt, gr);
+  sigma_adjoint(lam, psi, target_map(SL), gl, target_map(SR), gr);
 
   // 2. left chain: step n enlarges B_n with site n; B_n came from step n-1
   {
@@ -256,7 +266,7 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
         ex_->release(ob);
         break;
       }
-      AdjStep nx = make_step(*this, true, lb_[n - 1], n - 1);
+      AdjStep nx = adjoint_step(true, lb_[n - 1], n - 1);
       adj = back_renorm(nx, liso_[n - 1], lb_[n], ob);
       ex_->release(ob);
       cur = std::move(nx);
@@ -273,7 +283,7 @@ void Engine::integral_gradient(const double* lam, const double* psi, std::vector
         ex_->release(ob);
         break;
       }
-      AdjStep nx = make_step(*this, false, rb_[m + 2], m + 1);
+      AdjStep nx = adjoint_step(false, rb_[m + 2], m + 1);
       adj = back_renorm(nx, riso_[m + 1], rb_[m + 1], ob);
       ex_->release(ob);
       cur = std::move(nx);

@@ -390,8 +390,10 @@ void Engine::free_opset(OpSet& s) {
 
 void Engine::alloc_opset(OpSet& s) {
   int64_t n = 0;
+  int id = 0;
   for (auto& kv : s.ops)
     for (auto& b : kv.second.blk) {
+      b.id = id++;
       b.off = n;
       n += int64_t(b.rows) * b.cols;
     }
@@ -689,28 +691,85 @@ std::map<OpKey, EnlOpBuild<N>> collect_blocking(const Problem& P, bool left, con
 
 }  // namespace
 
-std::vector<BlockingTerm> Engine::blocking_terms(bool left, const Block& blk, int site, Enlarged& E) const {
-  std::map<OpKey, EnlOpBuild<Lin>> build = collect_blocking<Lin>(P_, left, blk, site, E);
-  std::vector<BlockingTerm> out;
-  for (auto& kv : build)
-    for (auto& tg : kv.second.tgt)
+AdjStep Engine::adjoint_step(bool left, const Block& blk, int site) const {
+  AdjStep st;
+  std::map<OpKey, EnlOpBuild<Lin>> build = collect_blocking<Lin>(P_, left, blk, site, st.E);
+  // every operator's list on its own (host threads), then side by side
+  struct Part {
+    std::vector<AdjTarget> tgt;
+    std::vector<AdjTerm> terms;
+    std::vector<std::pair<int64_t, double>> w;
+    int64_t n = 0;
+  };
+  std::vector<EnlOpBuild<Lin>*> ops;
+  for (auto& kv : build) {
+    st.keys.push_back(kv.first);
+    ops.push_back(&kv.second);
+  }
+  std::vector<Part> part(ops.size());
+  host_parallel_for(int(ops.size()), [&](int i) {
+    Part& p = part[size_t(i)];
+    std::vector<std::pair<int64_t, double>> m;
+    for (auto& tg : ops[size_t(i)]->tgt) {
+      AdjTarget t{i, tg.first.first, tg.first.second, p.n, int(p.terms.size()), 0};
       for (auto& pd : tg.second) {
-        BlockingTerm bt{kv.first, tg.first.first, tg.first.second, pd.src, pd.blk, pd.trans, Lin{pd.coef.c0, {}}};
-        // merge repeated integrals, drop zero weights
-        std::map<int64_t, double> w;
-        for (auto& x : pd.coef.w) w[x.first] += x.second;
-        for (auto& x : w)
-          if (x.second != 0.0) bt.coef.w.push_back(x);
-        out.push_back(std::move(bt));
+        AdjTerm x{pd.src, pd.blk, pd.trans, 0.0, int(p.w.size()), 0};
+        // repeated integrals merged (in the order they were added), zero weights dropped
+        m.assign(pd.coef.w.begin(), pd.coef.w.end());   // a handful: sorted by insertion
+        for (size_t k = 1; k < m.size(); ++k)
+          for (size_t j = k; j > 0 && m[j].first < m[j - 1].first; --j) std::swap(m[j], m[j - 1]);
+        for (size_t k = 0; k < m.size();) {
+          double s = 0.0;
+          const int64_t id = m[k].first;
+          for (; k < m.size() && m[k].first == id; ++k) s += m[k].second;
+          if (s != 0.0) p.w.push_back({id, s});
+        }
+        x.w1 = int(p.w.size());
+        const int64_t L2 = int64_t(P_.L) * P_.L;
+        double v = pd.coef.c0;
+        for (int k = x.w0; k < x.w1; ++k) {
+          const auto& w = p.w[size_t(k)];
+          v += w.second * (w.first < L2 ? P_.t[size_t(w.first)] : P_.v[size_t(w.first - L2)]);
+        }
+        x.val = v;
+        p.terms.push_back(x);
       }
-  return out;
-}
-
-double Engine::lin_value(const Lin& c) const {
-  const int64_t L2 = int64_t(P_.L) * P_.L;
-  double x = c.c0;
-  for (auto& w : c.w) x += w.second * (w.first < L2 ? P_.t[size_t(w.first)] : P_.v[size_t(w.first - L2)]);
-  return x;
+      t.t1 = int(p.terms.size());
+      p.n += int64_t(st.E.f_dim[t.rf]) * st.E.f_dim[t.cf];
+      p.tgt.push_back(t);
+    }
+    ops[size_t(i)]->tgt.clear();
+  });
+  std::vector<size_t> og(part.size() + 1, 0), ot(part.size() + 1, 0), ow(part.size() + 1, 0);
+  std::vector<int64_t> on(part.size() + 1, 0);
+  for (size_t i = 0; i < part.size(); ++i) {
+    og[i + 1] = og[i] + part[i].tgt.size();
+    ot[i + 1] = ot[i] + part[i].terms.size();
+    ow[i + 1] = ow[i] + part[i].w.size();
+    on[i + 1] = on[i] + part[i].n;
+  }
+  st.tgt.resize(og.back());
+  st.terms.resize(ot.back());
+  st.w.resize(ow.back());
+  st.n = on.back();
+  host_parallel_for(int(part.size()), [&](int i) {
+    const Part& p = part[size_t(i)];
+    for (size_t k = 0; k < p.tgt.size(); ++k) {
+      AdjTarget t = p.tgt[k];
+      t.off += on[size_t(i)];
+      t.t0 += int(ot[size_t(i)]);
+      t.t1 += int(ot[size_t(i)]);
+      st.tgt[og[size_t(i)] + k] = t;
+    }
+    for (size_t k = 0; k < p.terms.size(); ++k) {
+      AdjTerm t = p.terms[k];
+      t.w0 += int(ow[size_t(i)]);
+      t.w1 += int(ow[size_t(i)]);
+      st.terms[ot[size_t(i)] + k] = t;
+    }
+    std::copy(p.w.begin(), p.w.end(), st.w.begin() + std::ptrdiff_t(ow[size_t(i)]));
+  });
+  return st;
 }
 
 void Engine::enlarge(bool left, const Block& blk, int site, Enlarged& E, OpSet& out) {

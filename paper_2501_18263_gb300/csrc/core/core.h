@@ -105,6 +105,7 @@ struct OpBlk {
   int r, c;          // row / col sector (block sectors, or fine sectors on enlarged blocks)
   int rows, cols;
   int64_t off;       // element offset in the owning arena
+  int id = 0;        // number of the block in its operator set (alloc_opset)
   int ident = 0;     // enlarged only: block is c * identity (never read as a matrix)
   int64_t pn = -1, pt = -1;  // split-BF16 plane offsets: normal and transposed copies
 };
@@ -144,17 +145,31 @@ struct Site4T {
 };
 using Site4 = Site4T<double>;
 
-// One contribution of the blocking step, recorded for the adjoint: fine block
-// (rf, cf) of the enlarged operator `key` receives coef * (block src_blk of the
-// block operator src, transposed if trans; src == nullptr: the identity on the
-// block part) (x) a site-matrix entry, the entry and the Jordan-Wigner sign
-// folded into coef.
-struct BlockingTerm {
-  OpKey key;
-  int rf, cf;
+// The blocking step recorded for the adjoint, flat: every fine block of every enlarged
+// operator (a target, its adjoint at `off` of the step's arena) with its contributions,
+// targets in operator order, contributions in the order the forward build sums them.
+struct AdjTarget {
+  int key;            // index in AdjStep::keys
+  int rf, cf;         // fine block
+  int64_t off;
+  int t0, t1;         // its contributions
+};
+// fine block += coef * (block src_blk of the block operator src, transposed if trans;
+// src == nullptr: the identity on the block part) (x) a site-matrix entry, the entry and
+// the Jordan-Wigner sign folded into coef
+struct AdjTerm {
   const Op* src;
   int src_blk, trans;
-  Lin coef;
+  double val;         // coef for the present integrals
+  int w0, w1;         // coef's weights (integral index, weight), merged and nonzero
+};
+struct AdjStep {
+  Enlarged E;
+  std::vector<OpKey> keys;
+  std::vector<AdjTarget> tgt;
+  std::vector<AdjTerm> terms;
+  std::vector<std::pair<int64_t, double>> w;
+  int64_t n = 0;      // doubles of the step's adjoint arena
 };
 
 // One term of H_eff at a bond: c * op(L) (x) op(R), op = transpose if Lt / Rt,
@@ -276,8 +291,7 @@ class Engine {
   // the blocking steps and the renormalisations of both block chains.
   void integral_gradient(const double* lam, const double* psi, std::vector<double>& raw);
   // blocking contributions with their coefficients as linear forms (adjoint)
-  std::vector<BlockingTerm> blocking_terms(bool left, const Block& blk, int site, Enlarged& E) const;
-  double lin_value(const Lin& c) const;
+  AdjStep adjoint_step(bool left, const Block& blk, int site) const;
   // replace the integrals (chain order) and drop every block operator built from
   // the old ones; the loaded / swept isometries are kept
   void set_integrals(const std::vector<double>& t, const std::vector<double>& v);

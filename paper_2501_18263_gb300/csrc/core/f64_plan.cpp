@@ -61,21 +61,37 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
   const bool want_units = what & F64_UNITS, want_tiles = what & F64_TILES;
   F64PlanHost out;
   const int np = int(p.size());
-  // segments with K > 0, per problem
+  // segments with K > 0, per problem (the caller's list itself when it holds nothing else)
   std::vector<int> f0(size_t(np) + 1, 0);
-  std::vector<GemmSeg> seg;
-  seg.reserve(s.size());
   std::vector<int> use;   // problems with an output
   use.reserve(size_t(np));
-  for (int i = 0; i < np; ++i) {
-    f0[size_t(i)] = int(seg.size());
-    if (p[size_t(i)].M > 0 && p[size_t(i)].N > 0) {
-      use.push_back(i);
-      for (int k = p[size_t(i)].s0; k < p[size_t(i)].s1; ++k)
-        if (s[size_t(k)].K > 0) seg.push_back(s[size_t(k)]);
-    }
-    f0[size_t(i) + 1] = int(seg.size());
+  bool whole = true;
+  int at = 0;
+  for (int i = 0; i < np && whole; ++i) {
+    const GemmProb& q = p[size_t(i)];
+    whole = q.M > 0 && q.N > 0 && q.s0 == at;
+    for (int k = q.s0; k < q.s1; ++k) whole = whole && s[size_t(k)].K > 0;
+    f0[size_t(i)] = at;
+    at = q.s1;
   }
+  std::vector<GemmSeg> kept;
+  if (whole && at == int(s.size())) {
+    f0[size_t(np)] = at;
+    for (int i = 0; i < np; ++i) use.push_back(i);
+  } else {
+    kept.reserve(s.size());
+    for (int i = 0; i < np; ++i) {
+      f0[size_t(i)] = int(kept.size());
+      if (p[size_t(i)].M > 0 && p[size_t(i)].N > 0) {
+        use.push_back(i);
+        for (int k = p[size_t(i)].s0; k < p[size_t(i)].s1; ++k)
+          if (s[size_t(k)].K > 0) kept.push_back(s[size_t(k)]);
+      }
+    }
+    f0[size_t(np)] = int(kept.size());
+    whole = false;
+  }
+  const std::vector<GemmSeg>& seg = whole ? s : kept;
   if (use.empty()) return out;
 
   // 1. lists shared on the B side (rows stacked) and on the A side (columns stacked)

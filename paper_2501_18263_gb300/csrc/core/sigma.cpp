@@ -20,6 +20,7 @@
 #include <cstring>
 #include <stdexcept>
 #include <tuple>
+#include <unordered_map>
 
 #include "core.h"
 
@@ -269,6 +270,8 @@ void Engine::build_sigma_plan() {
     S.insert(S.end(), pp.S.begin(), pp.S.end());
   };
 
+  // only dmrg_davidson on an FP64 handle runs the plain form
+  const int forms = P_.precision == 0 ? GEMM_ANY | GEMM_PLAIN : GEMM_ANY;
   for (size_t ci = 0; ci < ranges.size(); ++ci) {
     const size_t n0 = ranges[ci].first, n1 = ranges[ci].second;
     std::vector<int64_t> xbase(T.size(), 0);
@@ -392,8 +395,8 @@ void Engine::build_sigma_plan() {
       st_.flops_stage2 += pp.flops;
     }
     Chunk ch;
-    ch.plan1 = P1.empty() ? -1 : ex_->gemm_plan(P1, S1);
-    ch.plan2 = ex_->gemm_plan(P2, S2);
+    ch.plan1 = P1.empty() ? -1 : ex_->gemm_plan(P1, S1, forms);
+    ch.plan2 = ex_->gemm_plan(P2, S2, forms);
     st_.n_gemm_problems += int(P1.size() + P2.size());
     st_.n_gemm_segments += int(S1.size() + S2.size());
     chunks_.push_back(ch);
@@ -428,7 +431,7 @@ void Engine::build_sigma_plan() {
         if (q.s1 > q.s0) P3.push_back(q);
       }
     }
-    plan_hl_ = P3.empty() ? -1 : ex_->gemm_plan(P3, S3);
+    plan_hl_ = P3.empty() ? -1 : ex_->gemm_plan(P3, S3, forms);
     st_.launches_per_sigma = (plan_hl_ >= 0 ? 1 : 0);
     for (auto& c : chunks_) st_.launches_per_sigma += (c.plan1 >= 0 ? 1 : 0) + 1;
     st_.n_gemm_problems += int(P3.size());
@@ -961,7 +964,7 @@ void Engine::build_sigma_plan() {
       PD.push_back(q);
     }
     ex_->diag(diag_tasks_);
-    diag_plan_ = ex_->gemm_plan(PD, SD);
+    diag_plan_ = ex_->gemm_plan(PD, SD, GEMM_PLAIN);
     ex_->gemm_run(diag_plan_, true);
   }
 }
@@ -1059,12 +1062,15 @@ void Engine::sigma_adjoint(const double* lam, const double* psi,
   for (auto& kv : EopsR_.ops) keyR[&kv.second] = kv.first;
   auto lcoarse = [&](const QN& q) { return EL.coarse.find(q); };
   auto rcoarse = [&](const QN& q) { return ER.coarse.find(q); };
-  auto target = [](const std::map<OpKey, std::map<std::pair<int, int>, int64_t>>& tm, const OpKey& k, int r,
-                   int c) -> int64_t {
+  using Fines = std::map<std::pair<int, int>, int64_t>;
+  auto fines_of = [](const std::map<OpKey, Fines>& tm, const OpKey& k) -> const Fines* {
     auto it = tm.find(k);
-    if (it == tm.end()) return -1;
-    auto jt = it->second.find({r, c});
-    return jt == it->second.end() ? -1 : jt->second;
+    return it == tm.end() ? nullptr : &it->second;
+  };
+  auto target = [](const Fines* m, int r, int c) -> int64_t {
+    if (!m) return -1;
+    auto jt = m->find({r, c});
+    return jt == m->end() ? -1 : jt->second;
   };
   const std::vector<Term> T = sigma_terms(true);
   struct XB { int iL, jR, iT, jT; int64_t off; };
@@ -1088,10 +1094,10 @@ void Engine::sigma_adjoint(const double* lam, const double* psi,
     xsize[n] = o;
   }
   std::vector<FineMap> fmL(T.size()), fmR(T.size());
-  for (size_t n = 0; n < T.size(); ++n) {
-    fmL[n] = fine_map(T[n].L);
-    fmR[n] = fine_map(T[n].R);
-  }
+  host_parallel_for(int(T.size()), [&](int n) {
+    fmL[size_t(n)] = fine_map(T[size_t(n)].L);
+    fmR[size_t(n)] = fine_map(T[size_t(n)].R);
+  });
   // chunks of terms: X and Y (each xsize) under the cap
   const int64_t cap = P_.mem_cap ? std::max<int64_t>(int64_t(1) << 14, int64_t(P_.mem_cap / 16 / sizeof(double)))
                                  : int64_t(1) << 27;
@@ -1121,16 +1127,18 @@ void Engine::sigma_adjoint(const double* lam, const double* psi,
     std::vector<GemmProb> P1;
     std::vector<GemmSeg> S1;
     // targets: C pointer -> (M, N, segments)
-    struct Acc { int M, N; std::vector<GemmSeg> segs; };
-    std::map<double*, Acc> acc;
+    struct Acc { double* C; int M, N; std::vector<GemmSeg> segs; };
+    std::vector<Acc> acc;
+    std::unordered_map<double*, int> where;
     auto add = [&](double* C, int M, int N, const GemmSeg& g) {
-      Acc& a = acc[C];
-      a.M = M;
-      a.N = N;
-      a.segs.push_back(g);
+      auto it = where.emplace(C, int(acc.size()));
+      if (it.second) acc.push_back(Acc{C, M, N, {}});
+      acc[size_t(it.first->second)].segs.push_back(g);
     };
     for (size_t n = rg.first; n < rg.second; ++n) {
       const Term& t = T[n];
+      const Fines* fl = t.L ? fines_of(tl, keyL.at(t.L)) : nullptr;
+      const Fines* fr = fines_of(tr, keyR.at(t.R));
       for (const XB& xb : xl[n]) {
         const int cols = ER.coarse.dim[xb.jR], colsT = ER.coarse.dim[xb.jT], rowsT = EL.coarse.dim[xb.iT];
         const QN qL = EL.coarse.q[xb.iL];
@@ -1182,30 +1190,28 @@ void Engine::sigma_adjoint(const double* lam, const double* psi,
             P1.push_back(q);
           }
           // L' operator: fine blocks (ft <- f), or (f <- ft) stored for a transposed use
-          const OpKey kl = keyL.at(t.L);
           for (int ft : EL.coarse_fines[xb.iT])
             for (int f : EL.coarse_fines[xb.iL]) {
               const double* Yr = Yb + int64_t(EL.f_row[ft]) * cols;
               const double* Pr = ps + int64_t(EL.f_row[f]) * cols;
               if (!t.Lt) {
-                const int64_t o = target(tl, kl, ft, f);
+                const int64_t o = target(fl, ft, f);
                 if (o >= 0) add(gl + o, EL.f_dim[ft], EL.f_dim[f], GemmSeg{Yr, Pr, cols, cols, cols, 0, 1});
               } else {
-                const int64_t o = target(tl, kl, f, ft);
+                const int64_t o = target(fl, f, ft);
                 if (o >= 0) add(gl + o, EL.f_dim[f], EL.f_dim[ft], GemmSeg{Pr, Yr, cols, cols, cols, 0, 1});
               }
             }
         }
         // R' operator: fine blocks (gt <- g), or (g <- gt) stored for a transposed use
-        const OpKey kr = keyR.at(t.R);
         for (int gt : ER.coarse_fines[xb.jT])
           for (int g : ER.coarse_fines[xb.jR]) {
             if (!t.Rt) {
-              const int64_t o = target(tr, kr, gt, g);
+              const int64_t o = target(fr, gt, g);
               if (o >= 0)
                 add(gr + o, ER.f_dim[gt], ER.f_dim[g], GemmSeg{lm + ER.f_row[gt], Xs + ER.f_row[g], colsT, cols, rowsT, 1, 0});
             } else {
-              const int64_t o = target(tr, kr, g, gt);
+              const int64_t o = target(fr, g, gt);
               if (o >= 0)
                 add(gr + o, ER.f_dim[g], ER.f_dim[gt], GemmSeg{Xs + ER.f_row[g], lm + ER.f_row[gt], cols, colsT, rowsT, 1, 0});
             }
@@ -1216,13 +1222,13 @@ void Engine::sigma_adjoint(const double* lam, const double* psi,
       // H_L' (x) 1: dF/dH_L'{ft <- f} = lam{i}[ft rows] psi{i}[f rows]^T
       const Op* HL = EopsL_.get(OP_H, 0);
       if (HL) {
-        const OpKey kh = keyL.at(HL);
+        const Fines* fh = fines_of(tl, keyL.at(HL));
         for (size_t i = 0; i < EL.coarse.q.size(); ++i) {
           if (psi_off_[i] < 0) continue;
           const int cols = ER.coarse.dim[psi_rcoarse_[i]];
           for (int ft : EL.coarse_fines[i])
             for (int f : EL.coarse_fines[i]) {
-              const int64_t o = target(tl, kh, ft, f);
+              const int64_t o = target(fh, ft, f);
               if (o < 0) continue;
               add(gl + o, EL.f_dim[ft], EL.f_dim[f],
                   GemmSeg{lam + psi_off_[i] + int64_t(EL.f_row[ft]) * cols, psi + psi_off_[i] + int64_t(EL.f_row[f]) * cols,
@@ -1234,16 +1240,16 @@ void Engine::sigma_adjoint(const double* lam, const double* psi,
     if (!P1.empty()) ex_->gemm(P1, S1);
     std::vector<GemmProb> P2;
     std::vector<GemmSeg> S2;
-    for (auto& kv : acc) {
+    for (const Acc& a : acc) {
       GemmProb q;
-      q.C = kv.first;
-      q.ldc = kv.second.N;
-      q.M = kv.second.M;
-      q.N = kv.second.N;
+      q.C = a.C;
+      q.ldc = a.N;
+      q.M = a.M;
+      q.N = a.N;
       q.alpha = 1.0;
       q.accumulate = 1;
       q.s0 = int(S2.size());
-      S2.insert(S2.end(), kv.second.segs.begin(), kv.second.segs.end());
+      S2.insert(S2.end(), a.segs.begin(), a.segs.end());
       q.s1 = int(S2.size());
       P2.push_back(q);
     }

@@ -120,6 +120,8 @@ struct SplitTask {
   uint16_t* dt;
 };
 
+enum { GEMM_ANY = 1, GEMM_PLAIN = 2 };
+
 class Exec {
  public:
   virtual ~Exec() {}
@@ -148,8 +150,9 @@ class Exec {
   // depend on the launch; otherwise the executor may use its tensor-core form (error
   // no larger, another rounding sequence)
   virtual void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain = false) = 0;
-  // persistent plans (uploaded once, replayed during Davidson)
-  virtual int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) = 0;
+  // persistent plans (uploaded once, replayed during Davidson); forms: what gemm_run may
+  // be asked for (GEMM_ANY: plain = false, GEMM_PLAIN: plain = true, or both)
+  virtual int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int forms) = 0;
   virtual void gemm_run(int plan, bool plain = false) = 0;
   virtual void plan_free(int plan) = 0;
   virtual void diag(const std::vector<DiagTask>& t) = 0;

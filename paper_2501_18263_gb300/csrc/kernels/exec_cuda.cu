@@ -789,39 +789,48 @@ class CudaExec : public Exec {
     bool live = false;
   };
 
-  int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) override {
-    return f64_plan(p, s, F64_UNITS | F64_TILES);
-  }
-  int f64_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int what) {
-    const F64PlanHost h = f64_build_plan(p, s, nsm_, what);
+  int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int forms) override {
+    const F64PlanHost h =
+        f64_build_plan(p, s, nsm_, (forms & GEMM_ANY ? F64_UNITS : 0) | (forms & GEMM_PLAIN ? F64_TILES : 0));
     Plan pl;
     pl.nunits = int(h.units.size());
     pl.nreds = int(h.reds.size());
     pl.ntiles = int(h.tiles.size());
     pl.npieces = h.pieces.empty() ? 0 : h.pieces.back();
-    // tables side by side, each at a multiple of 16 bytes; the two claim counters first
-    std::vector<char> buf(16, 0);
-    auto place = [&](const auto& v) {
-      const size_t at = buf.size(), n = v.size() * sizeof(v[0]);
-      buf.resize(at + ((n + 15) & ~size_t(15)));
-      if (n) std::memcpy(buf.data() + at, v.data(), n);
+    // tables side by side, each at a multiple of 16 bytes; the two claim counters first.
+    // Small plans go up in one copy, large ones table by table (one pass over them less)
+    size_t total = 16;
+    auto place = [&](size_t n) {
+      const size_t at = total;
+      total += (n + 15) & ~size_t(15);
       return at;
     };
-    buf.reserve(16 * 8 + sizeof(F64Unit) * (h.units.size() + h.tiles.size()) + sizeof(F64Row) * h.rows.size() +
-                sizeof(F64Ref) * (h.rowref.size() + h.colref.size()) + sizeof(F64Red) * h.reds.size() +
-                sizeof(int) * h.pieces.size());
-    const size_t o0 = place(h.units), o1 = place(h.rows), o2 = place(h.rowref), o3 = place(h.colref),
-                 o4 = place(h.reds), o5 = place(h.tiles), o6 = place(h.pieces);
-    char* d = reinterpret_cast<char*>(upload(buf));
+    const struct { const void* p; size_t n; } tab[7] = {
+        {h.units.data(), h.units.size() * sizeof(F64Unit)},   {h.rows.data(), h.rows.size() * sizeof(F64Row)},
+        {h.rowref.data(), h.rowref.size() * sizeof(F64Ref)},  {h.colref.data(), h.colref.size() * sizeof(F64Ref)},
+        {h.reds.data(), h.reds.size() * sizeof(F64Red)},      {h.tiles.data(), h.tiles.size() * sizeof(F64Unit)},
+        {h.pieces.data(), h.pieces.size() * sizeof(int)}};
+    size_t off[7];
+    for (int i = 0; i < 7; ++i) off[i] = place(tab[i].n);
+    char* d = static_cast<char*>(alloc(total));
+    if (total <= (size_t(1) << 20)) {
+      std::vector<char> buf(total, 0);
+      for (int i = 0; i < 7; ++i)
+        if (tab[i].n) std::memcpy(buf.data() + off[i], tab[i].p, tab[i].n);
+      h2d(d, buf.data(), total);
+    } else {
+      zero(d, 16);
+      for (int i = 0; i < 7; ++i) h2d(d + off[i], tab[i].p, tab[i].n);
+    }
     pl.mem = d;
     pl.next = reinterpret_cast<int*>(d);
-    pl.units = reinterpret_cast<F64Unit*>(d + o0);
-    pl.rows = reinterpret_cast<F64Row*>(d + o1);
-    pl.rowref = reinterpret_cast<F64Ref*>(d + o2);
-    pl.colref = reinterpret_cast<F64Ref*>(d + o3);
-    pl.reds = reinterpret_cast<F64Red*>(d + o4);
-    pl.tiles = reinterpret_cast<F64Unit*>(d + o5);
-    pl.pieces = reinterpret_cast<int*>(d + o6);
+    pl.units = reinterpret_cast<F64Unit*>(d + off[0]);
+    pl.rows = reinterpret_cast<F64Row*>(d + off[1]);
+    pl.rowref = reinterpret_cast<F64Ref*>(d + off[2]);
+    pl.colref = reinterpret_cast<F64Ref*>(d + off[3]);
+    pl.reds = reinterpret_cast<F64Red*>(d + off[4]);
+    pl.tiles = reinterpret_cast<F64Unit*>(d + off[5]);
+    pl.pieces = reinterpret_cast<int*>(d + off[6]);
     if (h.npart) pl.part = static_cast<double*>(alloc(sizeof(double) * size_t(h.npart)));
     pl.live = true;
     for (size_t i = 0; i < plans_.size(); ++i)
@@ -853,7 +862,7 @@ class CudaExec : public Exec {
   void plan_free(int id) override { free_plan_mem(plans_.at(id)); }
   void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain) override {
     if (p.empty()) return;
-    int id = f64_plan(p, s, plain ? F64_TILES : F64_UNITS);
+    int id = gemm_plan(p, s, plain ? GEMM_PLAIN : GEMM_ANY);
     gemm_run(id, plain);
     plan_free(id);
   }

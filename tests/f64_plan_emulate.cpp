@@ -16,6 +16,40 @@ struct Bad {};
 struct Octet { int s, k, n; };
 }  // namespace
 
+// The plain form (tiles): every element one chain of fused multiply-adds over its
+// segments and k.  Returns 0, or the code of the first broken rule.
+extern "C" int f64_emulate_plain(const GemmProb* p, int np, const GemmSeg* s, int ns, const double* lo,
+                                 const double* hi, int what) {
+  const F64PlanHost h = f64_build_plan(std::vector<GemmProb>(p, p + np), std::vector<GemmSeg>(s, s + ns), 4, what);
+  if (h.tiles.empty()) return 0;
+  if (h.pieces.size() != h.tiles.size() + 1) return 1;
+  for (size_t i = 0; i < h.tiles.size(); ++i) {
+    const F64Unit& u = h.tiles[i];
+    if (h.pieces[i + 1] - h.pieces[i] != (u.rows + F64_PR - 1) / F64_PR * ((u.nt + F64_PC - 1) / F64_PC)) return 2;
+    for (int r = 0; r < u.rows; ++r)
+      for (int c = 0; c < u.nt; ++c) {
+        int pos = u.pos0;
+        while (pos + 1 < u.pos0 + u.npos && h.rows[size_t(pos) + 1].pre <= u.row0 + r) ++pos;
+        const F64Row& R = h.rows[size_t(pos)];
+        const int m = u.row0 + r - R.pre;
+        if (m < 0 || m >= (R.m2 >> 1)) return 4;
+        double acc = 0;
+        for (int sg = 0; sg < u.nseg; ++sg) {
+          const F64Ref &a = h.rowref[size_t(R.s0 + sg)], &b = h.colref[size_t(u.cs + sg)];
+          for (int k = 0; k < (a.kt >> 1); ++k) {
+            const double* x = a.p + ((a.kt & 1) ? int64_t(k) * a.ld + m : int64_t(m) * a.ld + k);
+            const double* y = b.p + ((b.kt & 1) ? int64_t(k) * b.ld + u.n0 + c : int64_t(u.n0 + c) * b.ld + k);
+            if (x < lo || x >= hi || y < lo || y >= hi) return 6;
+            acc = std::fma(*x, *y, acc);
+          }
+        }
+        double* o = u.trans ? R.C + m + int64_t(u.n0 + c) * R.ldc : R.C + int64_t(m) * R.ldc + u.n0 + c;
+        *o = (R.m2 & 1) ? *o + R.alpha * acc : R.alpha * acc;
+      }
+  }
+  return 0;
+}
+
 // returns 0, or the code of the first broken rule; stat3 = units, reductions, log2 of
 // the largest digit sum among the weights that have to be exact
 extern "C" int f64_emulate(const GemmProb* p, int np, const GemmSeg* s, int ns, int nsm, const double* lo,

@@ -91,6 +91,22 @@ def _run(lib, ar, probs, out, nsm):
             (2.0 ** -52 * np.abs(old) if acc else 0) + 1e-300
         refs.append((co, ldc, M, N, ref, bound))
     S = (Seg * max(1, len(segs)))(*segs)
+    # the plain form, alone and with the other's stacking: the same bits
+    for what in (2, 3):
+        plain = out.copy()
+        Q = (Prob * len(probs))()
+        for i in range(len(probs)):
+            ctypes.memmove(ctypes.byref(Q[i]), ctypes.byref(P[i]), ctypes.sizeof(Prob))
+            Q[i].C = plain.ctypes.data + 8 * probs[i][0]
+        assert lib.f64_emulate_plain(Q, len(probs), S, len(segs), ctypes.c_void_p(ar.addr(0)),
+                                     ctypes.c_void_p(ar.addr(ar.a.size)), what) == 0
+        if what == 2:
+            first = plain
+        for co, ldc, M, N, ref, bound in refs:
+            if M and N:
+                got = plain[co:co + M * ldc].reshape(M, ldc)[:, :N]
+                assert np.all(np.abs(got - ref) <= bound)
+    assert np.array_equal(first, plain)
     stat = (ctypes.c_double * 3)()
     rc = lib.f64_emulate(P, len(probs), S, len(segs), nsm, ctypes.c_void_p(ar.addr(0)),
                          ctypes.c_void_p(ar.addr(ar.a.size)), stat)
