@@ -144,33 +144,41 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// one CTA per (range of elements, right-hand vector, group of MDOT_GRP vectors); every
+// product is summed over its threads and warps in the same order however the vectors
+// are grouped.  A group per CTA, not all vectors: with n in the thousands a launch had
+// two to four CTAs, each bound by the FP64 sums of 32 vectors (32 us at n = 4900,
+// m = 24; 6 us in groups of four)
+constexpr int MDOT_GRP = 4;
+
 __global__ void __launch_bounds__(256) mdot_partial(const double* __restrict__ V, int64_t ldv, int m,
                                                     const double* __restrict__ X, int64_t ldx, int64_t n,
                                                     double* __restrict__ part) {
-  const int j = blockIdx.y, b = blockIdx.x, nb = gridDim.x;
+  const int j = blockIdx.y, b = blockIdx.x, nb = gridDim.x, i0 = blockIdx.z * MDOT_GRP;
   const int64_t e0 = n * b / nb, e1 = n * (b + 1) / nb;
-  double acc[MDOT_MAX];
+  const int mg = min(MDOT_GRP, m - i0);
+  double acc[MDOT_GRP];
 #pragma unroll
-  for (int i = 0; i < MDOT_MAX; ++i) acc[i] = 0.0;
+  for (int i = 0; i < MDOT_GRP; ++i) acc[i] = 0.0;
   for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
     const double x = X[j * ldx + e];
 #pragma unroll
-    for (int i = 0; i < MDOT_MAX; ++i)
-      if (i < m) acc[i] = fma(V[i * ldv + e], x, acc[i]);
+    for (int i = 0; i < MDOT_GRP; ++i)
+      if (i < mg) acc[i] = fma(V[(i0 + i) * ldv + e], x, acc[i]);
   }
-  __shared__ double red[8][MDOT_MAX];
+  __shared__ double red[8][MDOT_GRP];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-  for (int i = 0; i < MDOT_MAX; ++i) {
-    if (i >= m) break;
+  for (int i = 0; i < MDOT_GRP; ++i) {
+    if (i >= mg) break;
     double s = warp_sum(acc[i]);
     if (l == 0) red[w][i] = s;
   }
   __syncthreads();
-  if (threadIdx.x < m) {
+  if (threadIdx.x < mg) {
     double s = 0.0;
     for (int ww = 0; ww < 8; ++ww) s += red[ww][threadIdx.x];
-    part[(int64_t(b) * gridDim.y + j) * MDOT_MAX + threadIdx.x] = s;
+    part[(int64_t(b) * gridDim.y + j) * MDOT_MAX + i0 + threadIdx.x] = s;
   }
 }
 
@@ -228,23 +236,26 @@ __device__ void jacobi_core(double* A, double* Z, int n, int ld, double* cs, int
   __syncthreads();
   for (int sweep = 0; sweep < 60; ++sweep) {
     // convergence: off-diagonal Frobenius norm relative to the full norm
+    // (summed by the first two warps, an order that does not depend on the CTA's size)
     double off = 0.0, tot = 0.0;
-    for (int e = tid; e < n * n; e += nt) {
+    for (int e = tid; e < n * n && tid < 64; e += 64) {
       const int i = e / n, j = e % n;
       const double a = A[i * ld + j];
       tot += a * a;
       if (i != j) off += a * a;
     }
-    off = warp_sum(off);
-    tot = warp_sum(tot);
-    if ((tid & 31) == 0) {
-      red[2 * (tid >> 5)] = off;
-      red[2 * (tid >> 5) + 1] = tot;
+    if (tid < 64) {
+      off = warp_sum(off);
+      tot = warp_sum(tot);
+      if ((tid & 31) == 0) {
+        red[2 * (tid >> 5)] = off;
+        red[2 * (tid >> 5) + 1] = tot;
+      }
     }
     __syncthreads();
     if (tid == 0) {
       double o = 0, t = 0;
-      for (int w = 0; w < nt / 32; ++w) {
+      for (int w = 0; w < 2; ++w) {
         o += red[2 * w];
         t += red[2 * w + 1];
       }
@@ -529,8 +540,12 @@ __global__ void __launch_bounds__(128) syev_perm_kernel(const SyevJob* jobs, con
   for (int row = threadIdx.x; row < n; row += blockDim.x) jb.Z[int64_t(row) * n + to] = src[row];
 }
 
-// Rayleigh-Ritz of the Davidson subspace: lowest eigenpair of an m x m matrix (m <= 40)
-__global__ void __launch_bounds__(64) ritz_kernel(const double* H, int ldh, int m, double* theta, double* y) {
+// Rayleigh-Ritz of the Davidson subspace: lowest eigenpair of an m x m matrix (m <= 40).
+// Eight warps: the rotations of a step are applied element by element on all four FP64
+// pipes of the SM (two warps used two of them)
+constexpr int RITZ_THREADS = 256;
+
+__global__ void __launch_bounds__(RITZ_THREADS) ritz_kernel(const double* H, int ldh, int m, double* theta, double* y) {
   __shared__ double A[40 * 40];
   __shared__ double Z[40 * 40];
   __shared__ double cs[44];
@@ -1118,7 +1133,7 @@ class CudaExec : public Exec {
     for (int i0 = 0; i0 < m; i0 += MDOT_MAX) {
       const int mm = std::min(MDOT_MAX, m - i0);
       const int nb = int(std::max<int64_t>(1, std::min<int64_t>((n + 4095) / 4096, 1024 / std::max(1, k))));
-      launch(PROF_VEC, [&] { mdot_partial<<<dim3(nb, k), 256, 0, st_>>>(V + i0 * ldv, ldv, mm, X, ldx, n, part_); });
+      launch(PROF_VEC, [&] { mdot_partial<<<dim3(nb, k, (mm + MDOT_GRP - 1) / MDOT_GRP), 256, 0, st_>>>(V + i0 * ldv, ldv, mm, X, ldx, n, part_); });
       launch(PROF_VEC, [&] { mdot_final<<<(mm * k + 127) / 128, 128, 0, st_>>>(part_, nb, mm, k, out + i0 * ldo, ldo); });
     }
   }
@@ -1137,7 +1152,7 @@ class CudaExec : public Exec {
   }
   void ritz(const double* H, int ldh, int m, double* theta, double* y) override {
     if (m > 40) throw std::runtime_error("ritz: subspace larger than 40");
-    launch(PROF_EIG, [&] { ritz_kernel<<<1, 64, 0, st_>>>(H, ldh, m, theta, y); });
+    launch(PROF_EIG, [&] { ritz_kernel<<<1, RITZ_THREADS, 0, st_>>>(H, ldh, m, theta, y); });
   }
   void syev(const std::vector<double*>& A, const std::vector<double*>& w, const std::vector<double*>& Z,
             const std::vector<int>& n) override {

@@ -68,15 +68,19 @@ __global__ void __launch_bounds__(32 * PLAIN_WARPS) gemm_f64_plain_kernel(
       nb = load_ref(rb + s + 1);
     }
   };
-  auto load = [&](double (&x)[8], double (&y)[8]) {
+  // the next batch's addresses and count; its elements are loaded one by one between
+  // the multiply-adds of the batch before, in the shadow of each other's pipe time
+  const double *qa = nullptr, *qb = nullptr;
+  int64_t ta = 0, tb = 0;
+  auto open = [&]() -> int {
+    if (s >= u.nseg) return 0;
+    qa = pa;
+    qb = pb;
+    ta = sa;
+    tb = sb;
     const int cnt = min(8, K - k);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {   // running pointers: a 64-bit multiply runs on the FP64 pipe
-      x[j] = j < cnt ? __ldg(pa) : 0.0;
-      y[j] = j < cnt ? __ldg(pb) : 0.0;
-      pa += sa;
-      pb += sb;
-    }
+    pa += 8 * sa;
+    pb += 8 * sb;
     k += 8;
     if (k >= K && ++s < u.nseg) enter();
     return cnt;
@@ -87,20 +91,25 @@ __global__ void __launch_bounds__(32 * PLAIN_WARPS) gemm_f64_plain_kernel(
     nb = load_ref(rb);
     enter();
     double x[8], y[8];
-    int cnt = load(x, y);
-    while (cnt > 0) {
-      double x1[8], y1[8];
-      int cnt1 = 0;
-      if (s < u.nseg) cnt1 = load(x1, y1);
+    int cnt = open();
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (j < cnt) acc = fma(x[j], y[j], acc);
+    for (int j = 0; j < 8; ++j) {
+      x[j] = j < cnt ? __ldg(qa) : 0.0;
+      y[j] = j < cnt ? __ldg(qb) : 0.0;
+      qa += ta;
+      qb += tb;
+    }
+    while (cnt > 0) {
+      const int next = open();
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        x[j] = x1[j];
-        y[j] = y1[j];
+        if (j < cnt) acc = fma(x[j], y[j], acc);
+        x[j] = j < next ? __ldg(qa) : 0.0;
+        y[j] = j < next ? __ldg(qb) : 0.0;
+        qa += ta;
+        qb += tb;
       }
-      cnt = cnt1;
+      cnt = next;
     }
   }
   if (!on) return;
