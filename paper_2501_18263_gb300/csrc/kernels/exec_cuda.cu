@@ -349,7 +349,7 @@ struct SyevJob {
   double* tau;    // n: reflector scalars
   double* Zc;     // n x n, column-major (Zc[c * n + r]): Q
   double* U;      // n x n: reflector k in row k (u_k[k + 1] = 1), then W = Q V (column-major)
-  double* pb;     // n: p = tau A22 v exchanged between the CTAs of a cluster
+  double* pb;     // 2 n: p = tau A22 v exchanged between the CTAs of a cluster
   int* perm;      // n: sorted position of eigenvalue i
   int n, pad;
 };
@@ -384,14 +384,18 @@ __device__ __forceinline__ int syev_find(const int* pre, int nj, int x) {
   return lo;
 }
 
-// step 1: a cluster of CS CTAs per matrix (CS = 1: one CTA).  Per column k every
-// CTA reads row k and forms the same reflector (the same reductions in the same
-// order); the rows of the trailing block are dealt out warp by warp over the
-// cluster for p = tau A22 v and for the rank-2 update, p is exchanged through
-// global scratch, and two cluster barriers per column order the steps (p complete
-// before it is read; the update complete before row k + 1 is read and before p is
-// overwritten).  The reflector goes to U (row k), so no CTA writes a row another
-// may still be reading.
+// step 1: a cluster of CS CTAs per matrix (CS = 1: one CTA).  The rank-2 update of step
+// k - 1 and the product p = tau A22 v of step k run in one pass over the trailing rows,
+// so that a column costs one cluster barrier (p complete; the rows updated) instead of
+// two and one read of the rows instead of two:
+//   every CTA forms row k after the pending update from the stored row and (v, w) of
+//   step k - 1, and from it the reflector v' (the same reductions in the same order);
+//   the rows of the trailing block are dealt out warp by warp over the cluster: row
+//   -= v_r w + w_r v, stored, and its product with v' taken in the same breath;
+//   p is exchanged through global scratch (two buffers in turn: a CTA may be a pass
+//   ahead of one that still reads), w' = p - (tau / 2) (p . v') v'.
+// A column of order about 300 takes 10 us of which 3 are FP64 arithmetic (eight CTAs);
+// the two-pass form took 19.
 __device__ __forceinline__ uint32_t syev_cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -410,18 +414,28 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
   const int n = jb.n;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
   extern __shared__ double sm[];
-  double* vs = sm;             // Householder vector of the current step
-  double* ps = vs + maxn;      // p = tau A22 v, then w
-  double* red = ps + maxn;     // 40 doubles: reductions and scalars
+  double* vs = sm;             // v and w of the step before (element i: row k + i), zero at first
+  double* ws = vs + maxn;
+  double* vn = ws + maxn;      // row k, then the reflector (element i: row k + 1 + i)
+  double* red = vn + maxn;     // 40 doubles: reductions and scalars
   double* A = jb.A;
+  for (int i = tid; i < n; i += nt) vs[i] = ws[i] = 0.0;
+  bool pending = false;
+  int par = 0;   // buffer of p: alternates over the columns that have a pass
+  __syncthreads();
   for (int k = 0; k + 2 < n; ++k) {
     const int m = n - k - 1;
-    const double* x = A + int64_t(k) * n + k + 1;    // row k right of the diagonal (= column k below it)
+    const double* row = A + int64_t(k) * n + k;
+    const double v0 = vs[0], w0 = ws[0];
     double part = 0.0;
-    for (int i = 1 + tid; i < m; i += nt) part += x[i] * x[i];
+    for (int i = 1 + tid; i <= m; i += nt) {
+      const double x = row[i] - (v0 * ws[i] + w0 * vs[i]);
+      vn[i - 1] = x;
+      if (i >= 2) part += x * x;
+    }
     const double sigma = block_sum(part, red);
     if (tid == 0) {
-      const double alpha = x[0];
+      const double alpha = vn[0];
       double beta = alpha, tau = 0.0, scale = 0.0;
       if (sigma != 0.0) {
         const double mu = sqrt(alpha * alpha + sigma);
@@ -432,58 +446,63 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
       red[34] = scale;
       red[35] = tau;
       if (rank == 0) {
-        jb.d[k] = A[int64_t(k) * n + k];
+        jb.d[k] = row[0] - (v0 * w0 + w0 * v0);
         jb.e[k] = beta;
         jb.tau[k] = tau;
       }
     }
     __syncthreads();
     const double tau = red[35], scale = red[34];
-    if (tau == 0.0) continue;   // H_k = I: A unchanged
+    if (tau == 0.0 && !pending) continue;   // H_k = I and A up to date
     double* u = jb.U + int64_t(k) * n + k + 1;
     for (int i = tid; i < m; i += nt) {
-      const double v = i == 0 ? 1.0 : x[i] * scale;
-      vs[i] = v;
+      const double v = tau == 0.0 ? 0.0 : i == 0 ? 1.0 : vn[i] * scale;
+      vn[i] = v;
       if (rank == 0) u[i] = v;   // the reflector, for step 2
     }
     __syncthreads();
-    // p = tau A22 v: one warp per row, rows dealt out over the cluster's warps
     double* A22 = A + int64_t(k + 1) * n + k + 1;
+    double* pb = jb.pb + par * n;
+    par ^= 1;
     for (int r = rank * nw + wid; r < m; r += CS * nw) {
-      const double* row = A22 + int64_t(r) * n;
+      double* a = A22 + int64_t(r) * n;
+      const double vr = vs[r + 1], wr = ws[r + 1];
       double acc = 0.0;
-      for (int j = lane; j < m; j += 32) acc += row[j] * vs[j];
-      acc = warp_sum(acc);
-      if (lane == 0) {
-        if (CS > 1) jb.pb[r] = tau * acc;
-        else ps[r] = tau * acc;
+      for (int j = lane; j < m; j += 32) {
+        const double x = a[j] - (vr * ws[j + 1] + wr * vs[j + 1]);
+        a[j] = x;
+        acc += x * vn[j];
       }
-    }
-    if (CS > 1) {
-      syev_cluster_sync();
-      for (int i = tid; i < m; i += nt) ps[i] = jb.pb[i];
-    }
-    __syncthreads();
-    double pv = 0.0;
-    for (int i = tid; i < m; i += nt) pv += ps[i] * vs[i];
-    const double K = 0.5 * tau * block_sum(pv, red);
-    for (int i = tid; i < m; i += nt) ps[i] -= K * vs[i];   // w
-    __syncthreads();
-    // A22 -= v w^T + w v^T on the same rows
-    for (int r = rank * nw + wid; r < m; r += CS * nw) {
-      double* row = A22 + int64_t(r) * n;
-      const double vr = vs[r], wr = ps[r];
-      for (int j = lane; j < m; j += 32) row[j] -= vr * ps[j] + wr * vs[j];
+      acc = warp_sum(acc);
+      if (lane == 0) pb[r] = tau * acc;
     }
     if (CS > 1) syev_cluster_sync();
     else __syncthreads();
+    // w' = p - (tau / 2) (p . v') v'
+    double pv = 0.0;
+    for (int i = tid; i < m; i += nt) {
+      const double p = __ldcg(pb + i);
+      ws[i] = p;
+      pv += p * vn[i];
+    }
+    const double K = 0.5 * tau * block_sum(pv, red);
+    for (int i = tid; i < m; i += nt) {
+      const double v = vn[i];
+      ws[i] -= K * v;
+      vs[i] = v;
+    }
+    pending = tau != 0.0;
+    __syncthreads();
   }
   if (tid == 0 && rank == 0) {
     if (n >= 2) {
-      jb.d[n - 2] = A[int64_t(n - 2) * n + n - 2];
-      jb.e[n - 2] = A[int64_t(n - 2) * n + n - 1];
+      const double* a = A + int64_t(n - 2) * n + n - 2;
+      jb.d[n - 2] = a[0] - (vs[0] * ws[0] + ws[0] * vs[0]);
+      jb.e[n - 2] = a[1] - (vs[0] * ws[1] + ws[0] * vs[1]);
+      jb.d[n - 1] = a[n + 1] - (vs[1] * ws[1] + ws[1] * vs[1]);
+    } else {
+      jb.d[n - 1] = A[0];
     }
-    jb.d[n - 1] = A[int64_t(n - 1) * n + n - 1];
     jb.e[n - 1] = 0.0;
   }
 }
@@ -1158,7 +1177,7 @@ class CudaExec : public Exec {
             const std::vector<int>& n) override {
     if (A.empty()) return;
     const int nj = int(A.size());
-    // per matrix: d, e, tau, pb (4n), Zc, U (2 n^2) doubles; perm (n) ints; every
+    // per matrix: d, e, tau, pb (5n), Zc, U (2 n^2) doubles; perm (n) ints; every
     // part 16-byte aligned
     auto up2 = [](int64_t x) { return (x + 1) & ~int64_t(1); };
     auto up4 = [](int64_t x) { return (x + 3) & ~int64_t(3); };
@@ -1171,13 +1190,13 @@ class CudaExec : public Exec {
       if (m <= 0) throw std::runtime_error("syev: empty matrix");
       if (m > 32767) throw std::runtime_error("syev: matrix order above 32767");
       doff[j] = dtot;
-      dtot += up2(4 * m) + 2 * up2(m * m);
+      dtot += up2(5 * m) + 2 * up2(m * m);
       ioff[j] = itot;
       itot += up4(m);
       pre_n[j + 1] = pre_n[j] + int(m);
       maxn = std::max(maxn, int(m) + 2);
     }
-    const size_t smem1 = sizeof(double) * (2 * size_t(maxn) + 40);
+    const size_t smem1 = sizeof(double) * (3 * size_t(maxn) + 40);
     if (smem1 > 227 * 1024) throw std::runtime_error("syev: matrix too large for the shared-memory workspace");
     double* dw = static_cast<double*>(alloc(sizeof(double) * size_t(dtot)));
     int* iw = static_cast<int*>(alloc(sizeof(int) * size_t(itot)));
@@ -1193,7 +1212,7 @@ class CudaExec : public Exec {
       jb.e = p + m;
       jb.tau = p + 2 * m;
       jb.pb = p + 3 * m;
-      p += up2(4 * m);
+      p += up2(5 * m);
       jb.Zc = p;
       p += up2(m * m);
       jb.U = p;
@@ -1201,10 +1220,12 @@ class CudaExec : public Exec {
       jb.n = int(m);
       jb.pad = 0;
     }
-    // 1. the reduction: a cluster of SYEV_CLUSTER CTAs for each matrix of order >= 256,
-    // one CTA for each smaller one; 2. Q
+    // 1. the reduction: a cluster of SYEV_CLUSTER CTAs for each matrix of order >= 80
+    // (largest first), one CTA for each smaller one, whose arithmetic one SM does in the
+    // time a cluster takes for its barriers; 2. Q
     std::vector<int> small, big;
-    for (int j = 0; j < nj; ++j) (n[j] >= 256 ? big : small).push_back(j);
+    for (int j = 0; j < nj; ++j) (n[j] >= 80 ? big : small).push_back(j);
+    std::stable_sort(big.begin(), big.end(), [&](int a, int b) { return n[size_t(a)] > n[size_t(b)]; });
     SyevJob* dj = upload(jobs);
     int* dpn = upload(pre_n);
     int* dsmall = upload(small);
