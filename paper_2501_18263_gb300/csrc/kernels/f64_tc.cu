@@ -195,26 +195,34 @@ struct Group {
   bool val;            // the row exists
 };
 
-// the lane's k pair in each of the B octets from o: all operand records first, then
-// all elements, so that a batch pays each of the two latencies once
+// the operand records of the B octets from o for the lane's row
 template <int B>
-__device__ __forceinline__ void load_octets(const Group& g, const int2* oct, int o, int kp, double (&x)[B][2]) {
-  F64Ref f[B];
+__device__ __forceinline__ void load_refs(const Group& g, const int2* oct, int o, int4 (&f)[B]) {
 #pragma unroll
-  for (int j = 0; j < B; ++j) {
-    const int4 v = __ldg(reinterpret_cast<const int4*>(g.ref + oct[o + j].x));
-    f[j].p = reinterpret_cast<const double*>((uint64_t(uint32_t(v.y)) << 32) | uint32_t(v.x));
-    f[j].ld = v.z;
-    f[j].kt = v.w;
-  }
+  for (int j = 0; j < B; ++j) f[j] = __ldg(reinterpret_cast<const int4*>(g.ref + oct[o + j].x));
+}
+
+// and the lane's k pair in each of them
+template <int B>
+__device__ __forceinline__ void load_pairs(const Group& g, const int2* oct, int o, int kp, const int4 (&f)[B],
+                                           double (&x)[B][2]) {
 #pragma unroll
   for (int j = 0; j < B; ++j) {
     const int e = oct[o + j].y, k = (e >> 4) + 2 * kp, n = g.val ? (e & 15) - 2 * kp : 0;
-    const bool t = f[j].kt & 1;
-    const double* p = f[j].p + (int64_t(t ? k : g.row) * f[j].ld + (t ? g.row : k));
+    const bool t = f[j].w & 1;
+    const double* p = reinterpret_cast<const double*>((uint64_t(uint32_t(f[j].y)) << 32) | uint32_t(f[j].x)) +
+                      (int64_t(t ? k : g.row) * f[j].z + (t ? g.row : k));
     x[j][0] = n > 0 ? __ldg(p) : 0.0;
-    x[j][1] = n > 1 ? __ldg(p + (t ? f[j].ld : 1)) : 0.0;
+    x[j][1] = n > 1 ? __ldg(p + (t ? f[j].z : 1)) : 0.0;
   }
+}
+
+// both, all records first, so that a batch pays each of the two latencies once
+template <int B>
+__device__ __forceinline__ void load_octets(const Group& g, const int2* oct, int o, int kp, double (&x)[B][2]) {
+  int4 f[B];
+  load_refs<B>(g, oct, o, f);
+  load_pairs<B>(g, oct, o, kp, f, x);
 }
 
 // the digits of two neighbouring elements of a row, digit w to address a + w stride:
@@ -370,17 +378,31 @@ __global__ void __maxnreg__(REGS)
       if (nOct > 0) {
         if (!mbar_wait_warp(ex_full(sl), ((chunk - 1) / SLOTS) & 1, abort_flag, err, 18)) break;
         const int ga = (S.rows + 7) >> 3, G8 = ga + ((S.nt + 7) >> 3), nst = (nOct + 1) >> 1;
-        // items (stage, group), the warp's next one loaded ahead
+        // items (stage, group): elements loaded one item ahead, operand records two
         int t = 0, g = warp, step0 = step;
+        auto next = [&](int& t, int& g) {
+          g += CONV;
+          while (g >= G8) {
+            g -= G8;
+            ++t;
+          }
+        };
         while (g >= G8) {
           g -= G8;
           ++t;
         }
-        Group q{};
+        int t1 = t, g1 = g;
+        next(t1, g1);
+        Group q{}, q1{};
+        int4 f1[2];
         double x[2][2];
         if (t < nst) {
           q = group(S, ga, g);
           load_octets<2>(q, S.oct, 2 * t, kp, x);
+        }
+        if (t1 < nst) {
+          q1 = group(S, ga, g1);
+          load_refs<2>(q1, S.oct, 2 * t1, f1);
         }
         int done = 0;   // stages this warp has arrived at
         while (!stop) {
@@ -402,27 +424,27 @@ __global__ void __maxnreg__(REGS)
             stop = true;
             break;
           }
-          // the next item
-          int t1 = t, g1 = g + CONV;
-          while (g1 >= G8) {
-            g1 -= G8;
-            ++t1;
-          }
-          Group q1 = q;
+          int t2 = t1, g2 = g1;
+          next(t2, g2);
           double y[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-          if (t1 < nst) {
-            q1 = group(S, ga, g1);
-            load_octets<2>(q1, S.oct, 2 * t1, kp, y);
+          if (t1 < nst) load_pairs<2>(q1, S.oct, 2 * t1, kp, f1, y);
+          Group q2 = q1;
+          if (t2 < nst) {
+            q2 = group(S, ga, g2);
+            load_refs<2>(q2, S.oct, 2 * t2, f1);
           }
           const int e = max(S.expo[q.ex] >> 20, 1);
           const uint32_t d = saddr(smem + st * STAGE_BYTES) + q.dst;
-          store_digits(x[0][0], x[0][1], e, d, q.dig);
-          store_digits(x[1][0], x[1][1], e, d + 128u, q.dig);
+#pragma unroll 1
+          for (int j = 0; j < 2; ++j)   // rolled: the loop body stays small for the instruction cache
+            store_digits(j ? x[1][0] : x[0][0], j ? x[1][1] : x[0][1], e, d + 128u * j, q.dig);
           q = q1;
+          q1 = q2;
 #pragma unroll
           for (int j = 0; j < 4; ++j) x[j >> 1][j & 1] = y[j >> 1][j & 1];
           t = t1;
-          g = g1;
+          t1 = t2;
+          g1 = g2;
         }
       }
       __syncwarp();
@@ -635,7 +657,8 @@ __global__ void __maxnreg__(REGS)
         ptrs[lane] = reinterpret_cast<uint64_t>(out) | (old ? 1u : 0u) | (ea == F64_SPECIAL ? 2u : 0u);
         __syncwarp();
       }
-      for (int cb = half * (n16 >> 1); cb < (half + 1) * (n16 >> 1) && cb < nt; cb += 8) {
+      // (a quarter without rows has nothing to do)
+      for (int cb = half * (n16 >> 1); cb < (half + 1) * (n16 >> 1) && cb < nt && quarter * 32 < nrows; cb += 8) {
         // a lane's column of the block, for the stores through shared memory
         const bool colsp = nOct > 0 && (S.expo[F64_TM + min(cb + (lane & 7), nt - 1)] >> 20) == F64_SPECIAL;
         if (__any_sync(0xffffffffu, ea == F64_SPECIAL || colsp)) {
