@@ -25,6 +25,7 @@ constexpr int F64_TM = 128;          // rows of a tile
 constexpr int F64_TN = 64;           // most columns of a tile
 constexpr int F64_CHUNK = 24;        // octets of a chunk
 constexpr int F64_PR = 8, F64_PC = 4;   // rows and columns of a piece
+constexpr int F64_LONG = 32;         // octets from which a plain sum counts as long
 
 // operand of one segment, seen from its side: element (r, k) at p[r ld + k] (kt even)
 // or p[k ld + r] (kt odd); K = kt / 2

@@ -357,15 +357,20 @@ struct SyevJob {
 constexpr int SYEV_THREADS = 1024;
 constexpr int SYEV_CLUSTER = 8;   // CTAs per large matrix in the reduction (portable cluster size)
 
-// sum over the CTA, returned to every thread (red: >= 33 doubles of shared memory)
-__device__ double block_sum(double v, double* red) {
-  v = warp_sum(v);
+// sum over the CTA, returned to every thread (red: >= 33 doubles of shared memory); only
+// the first `nv` threads hold terms, and only their warps add (FP64 adds of 32 warps of
+// zeros would take longer than the rest of a column's scalar work)
+__device__ double block_sum(double v, int nv, double* red) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int na = min(int(blockDim.x >> 5), (nv + 31) >> 5);
   __syncthreads();
-  if (lane == 0) red[w] = v;
+  if (w < na) {
+    v = warp_sum(v);
+    if (lane == 0) red[w] = v;
+  }
   __syncthreads();
   if (w == 0) {
-    double x = lane < int(blockDim.x >> 5) ? red[lane] : 0.0;
+    double x = lane < na ? red[lane] : 0.0;
     x = warp_sum(x);
     if (lane == 0) red[32] = x;
   }
@@ -429,11 +434,11 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
     const double v0 = vs[0], w0 = ws[0];
     double part = 0.0;
     for (int i = 1 + tid; i <= m; i += nt) {
-      const double x = row[i] - (v0 * ws[i] + w0 * vs[i]);
+      const double x = fma(-w0, vs[i], fma(-v0, ws[i], row[i]));
       vn[i - 1] = x;
       if (i >= 2) part += x * x;
     }
-    const double sigma = block_sum(part, red);
+    const double sigma = block_sum(part, m, red);
     if (tid == 0) {
       const double alpha = vn[0];
       double beta = alpha, tau = 0.0, scale = 0.0;
@@ -446,7 +451,7 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
       red[34] = scale;
       red[35] = tau;
       if (rank == 0) {
-        jb.d[k] = row[0] - (v0 * w0 + w0 * v0);
+        jb.d[k] = fma(-w0, v0, fma(-v0, w0, row[0]));
         jb.e[k] = beta;
         jb.tau[k] = tau;
       }
@@ -469,9 +474,9 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
       const double vr = vs[r + 1], wr = ws[r + 1];
       double acc = 0.0;
       for (int j = lane; j < m; j += 32) {
-        const double x = a[j] - (vr * ws[j + 1] + wr * vs[j + 1]);
+        const double x = fma(-wr, vs[j + 1], fma(-vr, ws[j + 1], a[j]));
         a[j] = x;
-        acc += x * vn[j];
+        acc = fma(x, vn[j], acc);
       }
       acc = warp_sum(acc);
       if (lane == 0) pb[r] = tau * acc;
@@ -485,7 +490,7 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
       ws[i] = p;
       pv += p * vn[i];
     }
-    const double K = 0.5 * tau * block_sum(pv, red);
+    const double K = 0.5 * tau * block_sum(pv, m, red);
     for (int i = tid; i < m; i += nt) {
       const double v = vn[i];
       ws[i] -= K * v;
@@ -497,9 +502,9 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
   if (tid == 0 && rank == 0) {
     if (n >= 2) {
       const double* a = A + int64_t(n - 2) * n + n - 2;
-      jb.d[n - 2] = a[0] - (vs[0] * ws[0] + ws[0] * vs[0]);
-      jb.e[n - 2] = a[1] - (vs[0] * ws[1] + ws[0] * vs[1]);
-      jb.d[n - 1] = a[n + 1] - (vs[1] * ws[1] + ws[1] * vs[1]);
+      jb.d[n - 2] = fma(-ws[0], vs[0], fma(-vs[0], ws[0], a[0]));
+      jb.e[n - 2] = fma(-ws[0], vs[1], fma(-vs[0], ws[1], a[1]));
+      jb.d[n - 1] = fma(-ws[1], vs[1], fma(-vs[1], ws[1], a[n + 1]));
     } else {
       jb.d[n - 1] = A[0];
     }
@@ -819,7 +824,7 @@ class CudaExec : public Exec {
     int* pieces = nullptr;
     int* next = nullptr;
     double* part = nullptr;
-    int nunits = 0, nreds = 0, ntiles = 0, npieces = 0;
+    int nunits = 0, nreds = 0, nlong = 0, plong = 0, ntiles = 0, npieces = 0;
     bool live = false;
   };
 
@@ -831,6 +836,8 @@ class CudaExec : public Exec {
     pl.nreds = int(h.reds.size());
     pl.ntiles = int(h.tiles.size());
     pl.npieces = h.pieces.empty() ? 0 : h.pieces.back();
+    while (pl.nlong < pl.ntiles && h.tiles[size_t(pl.nlong)].noct >= F64_LONG) ++pl.nlong;
+    pl.plong = pl.nlong ? h.pieces[size_t(pl.nlong)] : 0;
     // tables side by side, each at a multiple of 16 bytes; the two claim counters first.
     // Small plans go up in one copy, large ones table by table (one pass over them less)
     size_t total = 16;
@@ -880,7 +887,8 @@ class CudaExec : public Exec {
     if (!(plain ? pl.ntiles : pl.nunits)) return;
     launch(PROF_GEMM, [&] {
       if (plain) {
-        launch_gemm_f64_plain(pl.tiles, pl.pieces, pl.ntiles, pl.npieces, pl.rows, pl.rowref, pl.colref, st_);
+        launch_gemm_f64_plain(pl.tiles, pl.pieces, pl.nlong, pl.plong, pl.ntiles, pl.npieces, pl.rows, pl.rowref,
+                              pl.colref, err_, st_);
         return;
       }
       launch_gemm_f64_tc(pl.units, pl.nunits, pl.rows, pl.rowref, pl.colref, pl.part, pl.reds, pl.nreds, pl.next, err_, nsm_,

@@ -15,8 +15,10 @@ void launch_gemm_f64_tc(const F64Unit* units, int nunits, const F64Row* rows, co
                         cudaStream_t st);
 
 // the same problems by plain FP64 multiply-adds, every element's terms in the order of
-// its segments and k: tiles and the prefix sums of their pieces (npieces the last)
-void launch_gemm_f64_plain(const F64Unit* tiles, const int* pieces, int ntiles, int npieces, const F64Row* rows,
-                           const F64Ref* rowref, const F64Ref* colref, cudaStream_t st);
+// its segments and k: tiles (the first nlong, with plong pieces, are long sums) and the
+// prefix sums of their pieces (npieces the last)
+void launch_gemm_f64_plain(const F64Unit* tiles, const int* pieces, int nlong, int plong, int ntiles, int npieces,
+                           const F64Row* rows, const F64Ref* rowref, const F64Ref* colref, int* err,
+                           cudaStream_t st);
 
 }  // namespace dmrg
