@@ -55,6 +55,18 @@ inline int tile_of(int64_t n, int most, int unit) {
   return int(std::min<int64_t>(most, (w + unit - 1) / unit * unit));
 }
 
+// long sums first, the longest at the front; prefix sums of the tiles' pieces
+void order_tiles(F64PlanHost& out) {
+  const auto mid = std::stable_partition(out.tiles.begin(), out.tiles.end(),
+                                         [](const F64Unit& u) { return u.noct >= F64_LONG; });
+  std::stable_sort(out.tiles.begin(), mid, [](const F64Unit& a, const F64Unit& b) { return a.noct > b.noct; });
+  out.pieces.resize(out.tiles.size() + 1);
+  out.pieces[0] = 0;
+  for (size_t i = 0; i < out.tiles.size(); ++i)
+    out.pieces[i + 1] = out.pieces[i] + (out.tiles[i].rows + F64_PR - 1) / F64_PR *
+                                            ((out.tiles[i].nt + F64_PC - 1) / F64_PC);
+}
+
 }  // namespace
 
 F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int nsm, int what) {
@@ -94,6 +106,35 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
   const std::vector<GemmSeg>& seg = whole ? s : kept;
   if (use.empty()) return out;
 
+  // the plain form alone: every problem by itself, rows of A as rows
+  if (!want_units) {
+    out.rowref.resize(seg.size());
+    out.colref.resize(seg.size());
+    for (size_t k = 0; k < seg.size(); ++k) {
+      const GemmSeg& g = seg[k];
+      out.rowref[k] = F64Ref{g.A, g.lda, 2 * g.K + (g.ta ? 1 : 0)};
+      out.colref[k] = F64Ref{g.B, g.ldb, 2 * g.K + (g.tb ? 0 : 1)};
+    }
+    out.rows.reserve(use.size());
+    out.tiles.reserve(use.size());
+    for (int i : use) {
+      const GemmProb& q = p[size_t(i)];
+      F64Unit u{};
+      u.cs = f0[size_t(i)];
+      u.nseg = f0[size_t(i) + 1] - u.cs;
+      for (int k = u.cs; k < u.cs + u.nseg; ++k) u.noct += (seg[size_t(k)].K + 7) / 8;
+      u.pos0 = int(out.rows.size());
+      u.npos = 1;
+      u.part = -1;
+      out.rows.push_back(F64Row{q.C, q.alpha, q.ldc, u.cs, 0, 2 * q.M + (q.accumulate ? 1 : 0)});
+      u.rows = q.M;
+      u.nt = q.N;
+      out.tiles.push_back(u);
+    }
+    order_tiles(out);
+    return out;
+  }
+
   // 1. lists shared on the B side (rows stacked) and on the A side (columns stacked)
   auto same_b = [&](int i, int j) {
     if (p[size_t(i)].N != p[size_t(j)].N || f0[size_t(i) + 1] - f0[size_t(i)] != f0[size_t(j) + 1] - f0[size_t(j)])
@@ -130,7 +171,7 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     hashb[size_t(i)] = hb;
     hasha[size_t(i)] = ha;
   };
-  if (want_units) {
+  {
     const size_t work = use.size() + seg.size();
     if (work > 50000)
       host_parallel_for(nblk, [&](int b) {
@@ -165,15 +206,10 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     const double lanes = double((stack + F64_TM - 1) / F64_TM * F64_TM) / double(stack);
     return lanes * rows * double((cols + F64_TN - 1) / F64_TN) * tile_of(cols, F64_TN, 16);
   };
-  const int nb = want_units ? int(sumM.size()) : np;
+  const int nb = int(sumM.size());
   std::vector<int> grp(static_cast<size_t>(np), -1);
   std::vector<int> gcount(size_t(nb) + sumN.size(), 0);
   for (int i : use) {
-    if (!want_units) {
-      grp[size_t(i)] = i;
-      gcount[size_t(i)] = 1;
-      continue;
-    }
     const GemmProb& q = p[size_t(i)];
     const bool tr = share(q.N, sumN[size_t(ka[size_t(i)])], q.M) < share(q.M, sumM[size_t(kb[size_t(i)])], q.N);
     grp[size_t(i)] = tr ? nb + ka[size_t(i)] : kb[size_t(i)];
@@ -213,13 +249,14 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
   // schedulers) while the tensor core runs its 36 products; a chunk adds its pass for
   // the exponents and its drain, a unit its fixed latencies
   struct Tile { int g, pos0, npos, row0, rows, n0, nt; };
-  auto chunk_cost = [](int rows, int nt) {
+  auto part_cost = [](int rows, int nt, int64_t oct) {
     const double stage = std::max(28.0 * ((rows + 7) / 8 + (nt + 7) / 8), 18.0 * up16(nt));
-    return 12.0 * stage * 1.6 + 2500.0;
+    return 0.5 * double(oct) * stage * 1.6 + double((oct + F64_CHUNK - 1) / F64_CHUNK) * 2500.0 + 3000.0;
   };
   std::vector<Tile> tiles;
   std::vector<int64_t> goct(gorder.size(), 0);
   double total = 0;
+  int64_t chunks = 0;
   for (size_t gi = 0; gi < gorder.size(); ++gi) {
     const size_t g = size_t(gorder[gi]);
     const int m0 = gpos[g], m1 = m0 + gcount[g];
@@ -243,7 +280,6 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     for (int k = f0[size_t(i0)]; k < f0[size_t(i0) + 1]; ++k) oct += (seg[size_t(k)].K + 7) / 8;
     goct[gi] = oct;
     const int tm = tile_of(R, F64_TM, 8), tn = tile_of(cols, F64_TN, 16);
-    const int64_t nch = (oct + F64_CHUNK - 1) / F64_CHUNK;
     int pos = m0;
     for (int64_t r0 = 0; r0 < R; r0 += tm) {
       const int rows = int(std::min<int64_t>(tm, R - r0));
@@ -253,24 +289,26 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
       for (int n0 = 0; n0 < cols; n0 += tn) {
         const int nt = std::min(tn, cols - n0);
         tiles.push_back(Tile{int(gi), pos, last - pos + 1, int(r0), rows, n0, nt});
-        total += double(nch) * chunk_cost(rows, nt) + 3000.0;
+        total += part_cost(rows, nt, oct);
+        chunks += (oct + F64_CHUNK - 1) / F64_CHUNK;
       }
     }
   }
-  const double target = std::max(total / (4.0 * std::max(1, nsm)), 1.0);
+  // sums are cut at whole chunks, a small launch's at thirds of them (its time is one
+  // unit's latency: a chunk is twelve stages in a row)
+  const int gran = chunks < 4 * int64_t(nsm) ? F64_CHUNK / 3 : F64_CHUNK;
+  const double target = total / (4.0 * std::max(1, nsm));
   std::vector<F64Unit> units;
   std::vector<int> keys;
-  if (want_units) {
-    units.reserve(tiles.size());
-    keys.reserve(tiles.size());
-  }
+  units.reserve(tiles.size());
+  keys.reserve(tiles.size());
   if (want_tiles) out.tiles.reserve(tiles.size());
   for (const Tile& t : tiles) {
     const size_t g = size_t(gorder[size_t(t.g)]);
     const int m0 = gpos[g], i0 = member[size_t(m0)];
     const int cs = f0[size_t(i0)], nseg = f0[size_t(i0) + 1] - cs;
-    const int64_t oct = goct[size_t(t.g)], nch = (oct + F64_CHUNK - 1) / F64_CHUNK;
-    const double cc = chunk_cost(t.rows, t.nt);
+    const int64_t oct = goct[size_t(t.g)], nch = (oct + gran - 1) / gran;
+    const double cc = (part_cost(t.rows, t.nt, F64_CHUNK) - 3000.0) * gran / F64_CHUNK;
     const int64_t per = std::max<int64_t>(1, std::min<int64_t>(nch, int64_t(std::max(1.0, (target - 3000.0) / cc))));
     const int64_t parts = nch ? (nch + per - 1) / per : 1;
     F64Unit u{};
@@ -285,24 +323,23 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     u.trans = int(g) >= nb ? 1 : 0;
     u.part = -1;
     const int n16 = up16(t.nt);
-    if (want_units && parts > 1) {
+    if (parts > 1) {
       out.reds.push_back(F64Red{t.pos0, t.row0, t.rows, t.n0, t.nt, u.trans, int(parts), n16, out.npart});
     }
     int sg = 0, k0 = 0;
     u.noct = int(oct);
     if (want_tiles) out.tiles.push_back(u);
-    if (!want_units) continue;
     for (int64_t q = 0; q < parts; ++q) {
-      // whole chunks, spread evenly
+      // whole pieces of gran octets, spread evenly
       const int64_t c0 = nch * q / parts, c1 = nch * (q + 1) / parts;
       u.sg = sg;
       u.k0 = k0;
-      u.noct = int(std::min<int64_t>(c1 * F64_CHUNK, oct) - c0 * F64_CHUNK);
+      u.noct = int(std::min<int64_t>(c1 * gran, oct) - c0 * gran);
       if (parts > 1) {
         u.part = out.npart;
         out.npart += int64_t(F64_TM) * n16;
       }
-      const double cost = double(c1 - c0) * cc + 3000.0;
+      const double cost = part_cost(t.rows, t.nt, u.noct);
       units.push_back(u);
       keys.push_back(int(std::log2(cost) * 3.0));
       if (q + 1 < parts) {
@@ -323,7 +360,7 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
   }
   // longest first; units of about the same cost keep their order, so that tiles that
   // read the same operands run at the same time (a counting sort: few distinct keys)
-  if (want_units) {
+  {
     const int top = *std::max_element(keys.begin(), keys.end());
     std::vector<size_t> at(size_t(top) + 2, 0);
     for (int k : keys) ++at[size_t(top - k) + 1];
@@ -331,15 +368,7 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     out.units.resize(units.size());
     for (size_t i = 0; i < units.size(); ++i) out.units[at[size_t(top - keys[i])]++] = units[i];
   }
-  if (want_tiles) {
-    std::stable_sort(out.tiles.begin(), out.tiles.end(),
-                     [](const F64Unit& a, const F64Unit& b) { return a.noct > b.noct; });
-    out.pieces.reserve(out.tiles.size() + 1);
-    out.pieces.push_back(0);
-    for (const F64Unit& u : out.tiles)
-      out.pieces.push_back(out.pieces.back() +
-                           (u.rows + F64_PR - 1) / F64_PR * ((u.nt + F64_PC - 1) / F64_PC));
-  }
+  if (want_tiles) order_tiles(out);
   return out;
 }
 

@@ -11,7 +11,7 @@
 // K runs over all segments of a problem, in octets (8 consecutive k of one segment,
 // the last of a segment padded with zeros).  A chunk is at most 24 octets: up to 192 k
 // the digit sums of the weights that matter are exact in the tensor core's FP32
-// accumulators.  Long sums are split over units (ranges of whole chunks), whose
+// accumulators.  Long sums are split over units (ranges of octets), whose
 // partial sums are added in a fixed order by a second kernel.
 #pragma once
 #include <cstdint>
