@@ -69,6 +69,21 @@ void order_tiles(F64PlanHost& out) {
 
 }  // namespace
 
+bool f64_small(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) {
+  double mac = 0;
+  for (const GemmProb& q : p) {
+    int64_t len = 0, oct = 0;
+    for (int k = q.s0; k < q.s1; ++k) {
+      len += s[size_t(k)].K;
+      oct += (s[size_t(k)].K + 7) / 8;
+    }
+    if (len > F64_SMALL_K) return false;
+    mac += 8.0 * double(oct) * ((q.M + F64_PR - 1) / F64_PR * F64_PR) * ((q.N + F64_PC - 1) / F64_PC * F64_PC);
+    if (mac > F64_SMALL_MAC) return false;
+  }
+  return true;
+}
+
 F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int nsm, int what) {
   const bool want_units = what & F64_UNITS, want_tiles = what & F64_TILES;
   F64PlanHost out;

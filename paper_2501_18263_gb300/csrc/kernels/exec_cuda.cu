@@ -825,13 +825,16 @@ class CudaExec : public Exec {
     int* next = nullptr;
     double* part = nullptr;
     int nunits = 0, nreds = 0, nlong = 0, plong = 0, ntiles = 0, npieces = 0;
+    bool small = false;     // plain in any case
     bool live = false;
   };
 
   int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int forms) override {
-    const F64PlanHost h =
-        f64_build_plan(p, s, nsm_, (forms & GEMM_ANY ? F64_UNITS : 0) | (forms & GEMM_PLAIN ? F64_TILES : 0));
+    const bool small = f64_small(p, s);
+    const F64PlanHost h = f64_build_plan(
+        p, s, nsm_, (forms & GEMM_ANY && !small ? F64_UNITS : 0) | (forms & GEMM_PLAIN || small ? F64_TILES : 0));
     Plan pl;
+    pl.small = small;
     pl.nunits = int(h.units.size());
     pl.nreds = int(h.reds.size());
     pl.ntiles = int(h.tiles.size());
@@ -884,6 +887,7 @@ class CudaExec : public Exec {
   }
   void gemm_run(int id, bool plain) override {
     Plan& pl = plans_.at(id);
+    plain = plain || pl.small;
     if (!(plain ? pl.ntiles : pl.nunits)) return;
     launch(PROF_GEMM, [&] {
       if (plain) {

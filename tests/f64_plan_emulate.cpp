@@ -162,3 +162,18 @@ extern "C" int f64_emulate(const GemmProb* p, int np, const GemmSeg* s, int ns, 
   stat3[2] = top > 0 ? std::log2(top) : 0;
   return 0;
 }
+
+// the rule that sends a launch to the plain kernel, on sizes alone
+extern "C" int f64_emulate_small(int np, const int* M, const int* N, const int* nseg, int ns, const int* K) {
+  std::vector<GemmProb> p(static_cast<size_t>(np));
+  std::vector<GemmSeg> s(static_cast<size_t>(ns));
+  for (int k = 0; k < ns; ++k) s[size_t(k)].K = K[k];
+  int at = 0;
+  for (int i = 0; i < np; ++i) {
+    p[size_t(i)].M = M[i];
+    p[size_t(i)].N = N[i];
+    p[size_t(i)].s0 = at;
+    p[size_t(i)].s1 = at += nseg[i];
+  }
+  return f64_small(p, s) ? 1 : 0;
+}

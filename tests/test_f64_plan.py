@@ -186,3 +186,18 @@ def test_infinities_and_nan_propagate(lib):
     assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
     fine = np.isfinite(ref)
     assert np.allclose(got[fine], ref[fine], rtol=1e-13)
+
+
+@pytest.mark.parametrize("M, N, nseg, K, small", [
+    ([1], [1], [1], [512], 1),                       # the longest sum one warp keeps
+    ([1], [1], [1], [513], 0),
+    ([1, 1], [1, 1], [1, 2], [4, 256, 257], 0),      # over two segments
+    ([8] * 2, [4] * 2, [1, 0], [512], 1),            # an empty list
+    ([], [], [], [], 1),
+    ([8] * 366, [4] * 366, [1] * 366, [256] * 366, 1),    # 2 998 272 counted
+    ([8] * 367, [4] * 367, [1] * 367, [256] * 367, 0),    # 3 006 464
+    ([1] * 367, [1] * 367, [1] * 367, [249] * 367, 0),    # the same pieces and octets, ragged
+])
+def test_small_launches_are_plain(lib, M, N, nseg, K, small):
+    ints = [(ctypes.c_int * max(1, len(x)))(*x) for x in (M, N, nseg, K)]
+    assert lib.f64_emulate_small(len(M), ints[0], ints[1], ints[2], len(K), ints[3]) == small
