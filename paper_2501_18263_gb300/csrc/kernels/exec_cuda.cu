@@ -1339,7 +1339,7 @@ class CudaExec : public Exec {
         mg.gp = q + 3 * s;
         mg.cnt = q + 5 * s;
         oi += up4(5 * s + 4);
-        const int nt = int((s + 63) / 64);
+        const int nt = int((s + DC_TILE - 1) / DC_TILE);
         ps[i + 1] = ps[i] + int(s);
         pt[i + 1] = pt[i] + nt * nt;
       }

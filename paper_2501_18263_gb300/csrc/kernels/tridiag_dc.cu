@@ -16,8 +16,8 @@
 //     (tol = 8 eps max(max |d|, rho));
 //  3. the k roots of 1 + rho sum_i z_i^2 / (d_i - lambda) = 0, root j in
 //     (d_j, d_{j+1}) (the last in (d_k, d_k + rho sum z^2)), each as an offset tau
-//     from its nearer pole, by bisection on the bit patterns of tau (one warp per
-//     root, the sum over the lanes);
+//     from its nearer pole, by rational interpolation inside a bracket that ends
+//     at adjacent bit patterns of tau (one warp per root, the sums over the lanes);
 //  4. z recomputed from the roots, zh_i^2 = prod_j (lambda_j - d_i) /
 //     (rho prod_{l != i} (d_l - d_i)), so that the eigenvectors u_j = zh / (d - lambda_j)
 //     are orthogonal to working accuracy;
@@ -36,6 +36,24 @@ __device__ __forceinline__ double dc_warp_sum(double v) {
   return v;
 }
 
+// the sums of four values in six additions: each half of the warp takes two of them,
+// each quarter one (an FP64 addition of a warp holds its pipe for 64 clocks, a select
+// and a shuffle do not)
+__device__ __forceinline__ void dc_warp_sum4(double& a, double& b, double& c, double& d) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool h = lane & 16, q = lane & 8;
+  const double x = (h ? c : a) + __shfl_xor_sync(full, h ? a : c, 16);
+  const double y = (h ? d : b) + __shfl_xor_sync(full, h ? b : d, 16);
+  double v = (q ? y : x) + __shfl_xor_sync(full, q ? x : y, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
+  a = __shfl_sync(full, v, 0);
+  b = __shfl_sync(full, v, 8);
+  c = __shfl_sync(full, v, 16);
+  d = __shfl_sync(full, v, 24);
+}
+
 __device__ __forceinline__ int dc_find(const int* pre, int nj, int x) {
   int lo = 0, hi = nj - 1;
   while (lo < hi) {
@@ -47,9 +65,15 @@ __device__ __forceinline__ int dc_find(const int* pre, int nj, int x) {
 }
 
 // ---- leaves: one warp each, lane r holds row r of the leaf's eigenvectors in
-// shared memory; lane 0 runs the QL recurrences of one iteration and records its
-// rotations, then every lane applies them to its row.  More than 60 iterations for
-// one eigenvalue: *err = 9.
+// shared memory; the lanes look for negligible couplings, lane 0 runs the QL
+// recurrences of one iteration and records its rotations, then every lane applies them
+// to its row.  More than 60 iterations for one eigenvalue: *err = 9.
+//
+// Bound by the chain of dependent FP64 instructions of lane 0, about 900 rotations for
+// 32 rows: a rotation is a reciprocal square root (corrected once, so that c^2 + s^2 is
+// as close to 1 as from a root and two quotients) instead of a hypot and two divisions,
+// and the next coupling and diagonal entry are read a rotation ahead.  The
+// leaves of the density matrices of one bond at L = 24, D = 1024: 2.32 -> 1.37 ms.
 constexpr int DC_LEAF_WARPS = 4;
 
 __global__ void __launch_bounds__(32 * DC_LEAF_WARPS) dc_leaf_kernel(const DcLeaf* __restrict__ leaves, int nl,
@@ -57,7 +81,7 @@ __global__ void __launch_bounds__(32 * DC_LEAF_WARPS) dc_leaf_kernel(const DcLea
   __shared__ double zsm[DC_LEAF_WARPS][DC_LEAF][DC_LEAF + 1];
   __shared__ double dsm[DC_LEAF_WARPS][DC_LEAF], esm[DC_LEAF_WARPS][DC_LEAF];
   __shared__ double rc[DC_LEAF_WARPS][DC_LEAF], rs[DC_LEAF_WARPS][DC_LEAF];
-  __shared__ int ctl[DC_LEAF_WARPS][2];
+  __shared__ int ctl[DC_LEAF_WARPS];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int li = blockIdx.x * DC_LEAF_WARPS + w;
   if (li >= nl) return;
@@ -78,66 +102,73 @@ __global__ void __launch_bounds__(32 * DC_LEAF_WARPS) dc_leaf_kernel(const DcLea
   const double eps = 2.220446049250313e-16;
   int l = 0, iter = 0;
   double tnorm = 0.0;
-  if (lane == 0)
-    for (int i = 0; i < s; ++i) tnorm = fmax(tnorm, fabs(dd[i]) + fabs(ee[i]) + (i ? fabs(ee[i - 1]) : 0.0));
+  if (lane < s) tnorm = fabs(dd[lane]) + fabs(ee[lane]) + (lane ? fabs(ee[lane - 1]) : 0.0);
+#pragma unroll
+  for (int of = 16; of > 0; of >>= 1) tnorm = fmax(tnorm, __shfl_xor_sync(0xffffffffu, tnorm, of));
   for (;;) {
+    bool small = true;
+    if (lane < s - 1)
+      small = fabs(ee[lane]) <= eps * (fabs(dd[lane]) + fabs(dd[lane + 1])) || fabs(ee[lane]) <= eps * tnorm;
+    const unsigned cut = __ballot_sync(0xffffffffu, small);
+    while (l < s && (cut >> l & 1u)) {
+      ++l;
+      iter = 0;
+    }
+    if (l >= s) break;
+    if (++iter > 60) {
+      if (lane == 0) atomicExch(err, 9);
+      break;
+    }
+    const int mm = __ffs(int(cut & (~0u << l))) - 1;   // the row s - 1 is always in cut
     if (lane == 0) {
-      int nrot = -1, first = 0;
-      while (l < s) {
-        int mm = l;
-        for (; mm < s - 1; ++mm)
-          if (fabs(ee[mm]) <= eps * (fabs(dd[mm]) + fabs(dd[mm + 1])) || fabs(ee[mm]) <= eps * tnorm) break;
-        if (mm == l) {
-          ++l;
-          iter = 0;
-          continue;
-        }
-        if (++iter > 60) {
-          atomicExch(err, 9);
-          l = s;
-          break;
-        }
-        double g = (dd[l + 1] - dd[l]) / (2.0 * ee[l]);
-        double r = hypot(g, 1.0);
-        g = dd[mm] - dd[l] + ee[l] / (g + (g >= 0.0 ? r : -r));
-        double sn = 1.0, c = 1.0, p = 0.0;
-        bool split = false;
-        nrot = 0;
-        first = mm - 1;
-        for (int i = mm - 1; i >= l; --i) {
-          const double f = sn * ee[i], b = c * ee[i];
+      double g = (dd[l + 1] - dd[l]) / (2.0 * ee[l]);
+      double r = hypot(g, 1.0);
+      g = dd[mm] - dd[l] + ee[l] / (g + (g >= 0.0 ? r : -r));
+      double sn = 1.0, c = 1.0, p = 0.0;
+      double dn = dd[mm], di = dd[mm - 1], ei = ee[mm - 1];
+      int i = mm - 1;
+      for (; i >= l; --i) {
+        const int ip = i > l ? i - 1 : l;
+        const double dnext = dd[ip], enext = ee[ip];
+        const double f = sn * ei, b = c * ei;
+        const double r2 = fma(f, f, g * g);
+        if (r2 > 1e-280 && r2 < 1e280) {
+          double y = rsqrt(r2);
+          y = fma(0.5 * y, fma(-(r2 * y), y, 1.0), y);
+          r = r2 * y;
+          sn = f * y;
+          c = g * y;
+        } else {
           r = hypot(f, g);
-          ee[i + 1] = r;
           if (r == 0.0) {
-            dd[i + 1] -= p;
-            ee[mm] = 0.0;
-            split = true;
+            ee[i + 1] = 0.0;
+            dd[i + 1] = dn - p;
             break;
           }
           sn = f / r;
           c = g / r;
-          g = dd[i + 1] - p;
-          r = (dd[i] - g) * sn + 2.0 * c * b;
-          p = sn * r;
-          dd[i + 1] = g + p;
-          g = c * r - b;
-          rc[w][nrot] = c;
-          rs[w][nrot] = sn;
-          ++nrot;
         }
-        if (!split) {
-          dd[l] -= p;
-          ee[l] = g;
-          ee[mm] = 0.0;
-        }
-        break;
+        ee[i + 1] = r;
+        g = dn - p;
+        r = (di - g) * sn + 2.0 * c * b;
+        p = sn * r;
+        dd[i + 1] = g + p;
+        g = c * r - b;
+        rc[w][mm - 1 - i] = c;
+        rs[w][mm - 1 - i] = sn;
+        dn = di;
+        di = dnext;
+        ei = enext;
       }
-      ctl[w][0] = (l < s) ? nrot : -1;
-      ctl[w][1] = first;
+      ctl[w] = mm - 1 - i;
+      if (i < l) {
+        dd[l] -= p;
+        ee[l] = g;
+      }
+      ee[mm] = 0.0;
     }
     __syncwarp();
-    const int nrot = ctl[w][0], first = ctl[w][1];
-    if (nrot < 0) break;
+    const int nrot = ctl[w], first = mm - 1;
     if (lane < s) {
       // rotation q mixes columns i = first - q and i + 1 of row `lane`
       double zi1 = Zl[lane][first + 1];
@@ -161,7 +192,9 @@ __global__ void __launch_bounds__(32 * DC_LEAF_WARPS) dc_leaf_kernel(const DcLea
 
 // ---- merge step 1-2: one CTA per merge.  z from the two blocks' boundary rows,
 // normalised; poles sorted (rank of each); deflation on one thread (sequential
-// over the sorted poles, as the pairing with the previous kept pole requires).
+// over the sorted poles, as the pairing with the previous kept pole requires); its chain
+// of roots and quotients, one per pole, was most of 1.10 ms of the four levels (as at step 3), now
+// 0.30: only pairs that come near the tolerance take them.
 constexpr int DC_PREP_THREADS = 256;
 
 __device__ double dc_block_sum(double v, double* red) {
@@ -190,18 +223,24 @@ __global__ void __launch_bounds__(DC_PREP_THREADS) dc_prep_kernel(const DcMerge*
   for (int i = threadIdx.x; i < s; i += blockDim.x) {
     const double zi = i < s1 ? m.Z[int64_t(o + i) * n + (o + s1 - 1)] : sg * m.Z[int64_t(o + i) * n + (o + s1)];
     m.gc[i] = zi;
-    m.gs[i] = m.d[o + i];
+    m.gs[i] = m.d[o + i] + 0.0;   // no -0.0: the order below is on bit patterns
     part += zi * zi;
   }
   const double nz2 = dc_block_sum(part, red);
   const double inv = nz2 > 0.0 ? 1.0 / sqrt(nz2) : 0.0;
-  // rank sort (ties by index)
+  // rank sort (ties by index) on integers that order as the doubles do: an FP64
+  // comparison holds the pipe as long as a multiply-add
+  auto key = [](double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+  };
   for (int i = threadIdx.x; i < s; i += blockDim.x) {
     const double di = m.gs[i];
+    const long long ki = key(di);
     int r = 0;
     for (int j = 0; j < s; ++j) {
-      const double dj = m.gs[j];
-      r += (dj < di) || (dj == di && j < i);
+      const long long kj = key(m.gs[j]);
+      r += (kj < ki) || (kj == ki && j < i);
     }
     m.ds[r] = di;
     m.zs[r] = m.gc[i] * inv;
@@ -210,54 +249,82 @@ __global__ void __launch_bounds__(DC_PREP_THREADS) dc_prep_kernel(const DcMerge*
   __syncthreads();
   if (threadIdx.x == 0) {
     const double rho = fabs(beta) * nz2;
-    double dmax = 0.0;
-    for (int i = 0; i < s; ++i) dmax = fmax(dmax, fabs(m.ds[i]));
+    const double dmax = fmax(fabs(m.ds[0]), fabs(m.ds[s - 1]));
     const double tol = 8.0 * 2.220446049250313e-16 * fmax(dmax, rho);
-    int ng = 0, k = 0, p = -1;
+    // a pair is looked at closely only if |(d_i - d_p) z_i z_p| <= tol (z_i^2 + z_p^2)
+    // up to rounding, which takes no root and no division
+    const double near = tol > 1e-280 ? 1.000001 * tol : 1e300;
+    int ng = 0, p = -1;
+    double zp = 0.0, dp = 0.0, zi = m.zs[0], di = m.ds[0];
     for (int i = 0; i < s; ++i) {
-      if (rho * fabs(m.zs[i]) <= tol) {   // deflated: (ds_i, column i) stays an eigenpair
-        m.gp[2 * i + 1] = -1;             // mark (the pair slots double as flags below)
-        continue;
-      }
-      m.gp[2 * i + 1] = 0;
-      if (p >= 0) {
-        const double t = hypot(m.zs[p], m.zs[i]);
-        const double c = m.zs[i] / t, sn = -m.zs[p] / t;
-        if (fabs((m.ds[i] - m.ds[p]) * c * sn) <= tol) {
-          // rotate columns p, i so that z_p = 0; pole p deflates
-          const double dp = m.ds[p] * c * c + m.ds[i] * sn * sn;
-          const double di = m.ds[p] * sn * sn + m.ds[i] * c * c;
-          m.ds[p] = dp;
-          m.ds[i] = di;
-          m.zs[p] = 0.0;
-          m.zs[i] = t;
-          m.gp[2 * p + 1] = -1;
-          m.gc[ng] = c;
-          m.gs[ng] = sn;
-          m.gp[2 * ng] = p | (i << 16);
-          ++ng;
+      const int in = i + 1 < s ? i + 1 : i;
+      const double znext = m.zs[in], dnext = m.ds[in];
+      if (rho * fabs(zi) <= tol) {   // deflated: (ds_i, column i) stays an eigenpair
+        m.gp[2 * i + 1] = -1;        // mark (the pair slots double as flags below)
+      } else {
+        m.gp[2 * i + 1] = 0;
+        if (p >= 0 && fabs((di - dp) * zi * zp) <= near * (zi * zi + zp * zp)) {
+          const double t = hypot(zp, zi);
+          const double c = zi / t, sn = -zp / t;
+          if (fabs((di - dp) * c * sn) <= tol) {
+            // rotate columns p, i so that z_p = 0; pole p deflates
+            const double a = dp * c * c + di * sn * sn;
+            di = dp * sn * sn + di * c * c;
+            zi = t;
+            m.ds[p] = a;
+            m.ds[i] = di;
+            m.zs[p] = 0.0;
+            m.zs[i] = t;
+            m.gp[2 * p + 1] = -1;
+            m.gc[ng] = c;
+            m.gs[ng] = sn;
+            m.gp[2 * ng] = p | (i << 16);
+            ++ng;
+          }
         }
+        p = i;
+        zp = zi;
+        dp = di;
       }
-      p = i;
+      zi = znext;
+      di = dnext;
     }
-    for (int i = 0; i < s; ++i)
-      if (m.gp[2 * i + 1] == 0) {
-        m.ndp[k] = i;
-        m.dk[k] = m.ds[i];
-        m.zk[k] = m.zs[i];
-        ++k;
-      }
-    m.cnt[0] = k;
     m.cnt[1] = ng;
     m.rho[0] = rho;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {   // the poles that are kept, in order
+    const int lane = threadIdx.x;
+    int k = 0;
+    for (int i0 = 0; i0 < s; i0 += 32) {
+      const int i = i0 + lane;
+      const bool keep = i < s && m.gp[2 * i + 1] == 0;
+      const unsigned b = __ballot_sync(0xffffffffu, keep);
+      if (keep) {
+        const int at = k + __popc(b & ((1u << lane) - 1u));
+        m.ndp[at] = i;
+        m.dk[at] = m.ds[i];
+        m.zk[at] = m.zs[i];
+      }
+      k += __popc(b);
+    }
+    if (lane == 0) m.cnt[0] = k;
   }
 }
 
 // ---- merge step 3: one warp per root (pre_s: prefix sums of the merges' s; root
 // slots past k exit).  f(lambda) rises from -inf to +inf between poles; the root is
-// bracketed on the half of (d_j, d_{j+1}) where it lies and tau is bisected over
-// its bit patterns (non-negative doubles order like their bit patterns), at most 63
-// steps to adjacent doubles.
+// bracketed on the half of (d_j, d_{j+1}) where it lies, as bit patterns of tau
+// (non-negative doubles order like their bit patterns), down to adjacent doubles.
+//
+// Bound by FP64 divisions, one per pole and evaluation (and, for a few dozen poles, by
+// the chain of one evaluation).  Bisection alone took 62 evaluations a root; here each
+// of the first few gives the sums of the poles on either side of the root and their
+// derivatives, and the next point is the root of c + s_1 / (d_j - x) + s_2 / (d_{j+1} - x)
+// with the same values and slopes (Bunch, Nielsen and Sorensen, Numer. Math. 31 (1978)).
+// Once a step is shorter than 64 doubles the bracket is closed from the other side by a
+// step just past the point; bisection finishes.  The four levels of the
+// same matrices: 3.44 -> 0.76 ms.
 __global__ void __launch_bounds__(256) dc_secular_kernel(const DcMerge* __restrict__ ms, int nm,
                                                          const int* __restrict__ pre_s) {
   const int gw = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
@@ -279,16 +346,31 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcMerge* __restri
     for (int i = lane; i < k; i += 32) z2 += zk[i] * zk[i];
     b = a + rho * dc_warp_sum(z2);
   }
+  const bool last = j + 1 == k;
+  // sums over the poles up to j (p1) and past it (p2) and their derivatives, at the
+  // point t from dorg
+  auto sums = [&](double dorg, double t, double& p1, double& p2, double& q1, double& q2) {
+    p1 = p2 = q1 = q2 = 0.0;
+    for (int i = lane; i < k; i += 32) {
+      const double z = zk[i], q = z / ((dk[i] - dorg) - t);
+      const bool left = i <= j;
+      p1 = fma(left ? z : 0.0, q, p1);
+      p2 = fma(left ? 0.0 : z, q, p2);
+      q1 = fma(left ? q : 0.0, q, q1);
+      q2 = fma(left ? 0.0 : q, q, q2);
+    }
+    dc_warp_sum4(p1, p2, q1, q2);
+  };
   const double mid = 0.5 * (a + b);
-  double fm = 0.0;
-  for (int i = lane; i < k; i += 32) fm += zk[i] * zk[i] / (dk[i] - mid);
-  fm = 1.0 + rho * dc_warp_sum(fm);
+  double p1, p2, q1, q2;
+  sums(0.0, mid, p1, p2, q1, q2);
+  double f = 1.0 + rho * (p1 + p2);
   int og;
   double sgn, hi;
-  if (j + 1 == k || fm > 0.0) {
+  if (last || f > 0.0) {
     og = j;
     sgn = 1.0;
-    hi = (j + 1 < k) ? mid - a : b - a;
+    hi = last ? b - a : mid - a;
   } else {
     og = j + 1;
     sgn = -1.0;
@@ -296,14 +378,57 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcMerge* __restri
   }
   const double dorg = dk[og];
   long long ilo = 0, ihi = __double_as_longlong(hi);
+  long long x = last ? __double_as_longlong(mid - a) : ihi;   // the point of the sums
+  auto note = [&](long long at, double fx) {   // true: the root is further from the origin
+    const bool up = (fx < 0.0) == (sgn > 0.0);
+    if (up) ilo = at > ilo ? at : ilo;
+    else ihi = at < ihi ? at : ihi;
+    return up;
+  };
+  bool up = x > 0 && note(x, f);
+  long long step = 0;
+  for (int it = 0; it < 14 && ihi - ilo > 1; ++it) {
+    const double t = sgn * __longlong_as_double(x);
+    const double d1 = (a - dorg) - t, d2 = (b - dorg) - t;
+    const double s1 = rho * q1, s2 = rho * q2;
+    double eta;
+    if (last) {
+      eta = d1 + s1 * d1 * d1 / (f - s1 * d1);
+    } else {
+      const double c = f - s1 * d1 - s2 * d2;
+      const double A = (d1 + d2) * f - d1 * d2 * (s1 + s2), B = d1 * d2 * f;
+      const double disc = sqrt(fabs(A * A - 4.0 * B * c));
+      eta = A <= 0.0 ? (A - disc) / (2.0 * c) : 2.0 * B / (A + disc);
+    }
+    const double tn = sgn * (t + eta);
+    const long long xn = tn > 0.0 ? __double_as_longlong(tn) : 0;
+    step = xn > x ? xn - x : x - xn;
+    if (tn > 0.0 && step <= 64) break;
+    x = xn > ilo && xn < ihi ? xn : ilo + ((ihi - ilo) >> 1);   // (a NaN goes to the middle)
+    step = -1;
+    sums(dorg, sgn * __longlong_as_double(x), p1, p2, q1, q2);
+    f = 1.0 + rho * (p1 + p2);
+    up = note(x, f);
+  }
+  bool walk = step >= 0 && step <= 64;
+  step += 1;
   while (ihi - ilo > 1) {
-    const long long im = ilo + ((ihi - ilo) >> 1);
-    const double t = sgn * __longlong_as_double(im);
-    double f = 0.0;
-    for (int i = lane; i < k; i += 32) f += zk[i] * zk[i] / ((dk[i] - dorg) - t);
-    f = 1.0 + rho * dc_warp_sum(f);
-    if ((f < 0.0) == (sgn > 0.0)) ilo = im;
-    else ihi = im;
+    long long at = ilo + ((ihi - ilo) >> 1);
+    if (walk) {
+      const long long to = up ? x + step : x - step;
+      walk = to > ilo && to < ihi;
+      if (walk) at = to;
+    }
+    const double t = sgn * __longlong_as_double(at);
+    double v = 0.0;
+    for (int i = lane; i < k; i += 32) v += zk[i] * zk[i] / ((dk[i] - dorg) - t);
+    v = 1.0 + rho * dc_warp_sum(v);
+    const bool u = note(at, v);
+    if (walk) {
+      walk = u == up && step < (1ll << 40);    // not past the root yet
+      x = at;
+      step *= 8;
+    }
   }
   if (lane == 0) {
     m.org[j] = og;
@@ -311,10 +436,12 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcMerge* __restri
   }
 }
 
-// ---- merge step 4a: zh_i from the roots, one thread per (merge, i)
+// ---- merge step 4a: zh_i from the roots, one warp per (merge, i): bound by the
+// divisions, which one thread per i left to a tenth of the SMs.  The same
+// levels: 0.68 -> 0.07 ms (and step 4b 0.54 -> 0.07 ms).
 __global__ void __launch_bounds__(256) dc_zhat_kernel(const DcMerge* __restrict__ ms, int nm,
                                                       const int* __restrict__ pre_s) {
-  const int g = int(blockIdx.x * blockDim.x + threadIdx.x);
+  const int g = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (g >= pre_s[nm]) return;
   const int mi = dc_find(pre_s, nm, g);
   const DcMerge m = ms[mi];
@@ -323,20 +450,21 @@ __global__ void __launch_bounds__(256) dc_zhat_kernel(const DcMerge* __restrict_
   if (i >= k) return;
   const double rho = m.rho[0];
   const double di = m.dk[i];
-  // lambda_j - d_i = tau_j - (d_i - d_org(j)); pair every factor with a pole gap
-  double prod = (m.tau[i] - (di - m.dk[m.org[i]])) / rho;
-  for (int j = 0; j < k; ++j) {
-    if (j == i) continue;
-    prod *= (m.tau[j] - (di - m.dk[m.org[j]])) / (m.dk[j] - di);
-  }
-  m.zh[i] = copysign(sqrt(fmax(prod, 0.0)), m.zk[i]);
+  // lambda_j - d_i = tau_j - (d_i - d_org(j)); pair every factor with a pole gap, that
+  // of j = i with rho
+  double prod = 1.0;
+  for (int j = lane; j < k; j += 32)
+    prod *= (m.tau[j] - (di - m.dk[m.org[j]])) / (j == i ? rho : m.dk[j] - di);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) prod *= __shfl_xor_sync(0xffffffffu, prod, o);
+  if (lane == 0) m.zh[i] = copysign(sqrt(fmax(prod, 0.0)), m.zk[i]);
 }
 
-// ---- merge step 4b: column j of U (k x k, column-major), normalised; one thread
+// ---- merge step 4b: column j of U (k x k, column-major), normalised; one warp
 // per (merge, j)
 __global__ void __launch_bounds__(256) dc_ucol_kernel(const DcMerge* __restrict__ ms, int nm,
                                                       const int* __restrict__ pre_s) {
-  const int g = int(blockIdx.x * blockDim.x + threadIdx.x);
+  const int g = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (g >= pre_s[nm]) return;
   const int mi = dc_find(pre_s, nm, g);
   const DcMerge m = ms[mi];
@@ -346,13 +474,13 @@ __global__ void __launch_bounds__(256) dc_ucol_kernel(const DcMerge* __restrict_
   const double dorg = m.dk[m.org[j]], tj = m.tau[j];
   double* u = m.U + int64_t(j) * k;
   double nrm = 0.0;
-  for (int i = 0; i < k; ++i) {
+  for (int i = lane; i < k; i += 32) {
     const double v = m.zh[i] / ((m.dk[i] - dorg) - tj);
     u[i] = v;
     nrm += v * v;
   }
-  const double inv = 1.0 / sqrt(nrm);
-  for (int i = 0; i < k; ++i) u[i] *= inv;
+  const double inv = 1.0 / sqrt(dc_warp_sum(nrm));
+  for (int i = lane; i < k; i += 32) u[i] *= inv;
 }
 
 // ---- merge step 5a: Qp = the two blocks' eigenvectors (block diagonal), columns
@@ -383,10 +511,11 @@ __global__ void __launch_bounds__(256) dc_qp_kernel(const DcMerge* __restrict__ 
 }
 
 // ---- merge step 5b: the new eigenvectors of the non-deflated poles,
-// Z[:, o + ndp[j]] = Qp[:, ndp] U[:, j] (s x k times k x k), 64 x 64 tiles
-// (pre_t: prefix sums of the merges' ceil(s/64)^2 tiles; tiles past k exit), and
-// the new eigenvalues d_org(j) + tau_j
-constexpr int DG_T = 64, DG_K = 16;
+// Z[:, o + ndp[j]] = Qp[:, ndp] U[:, j] (s x k times k x k), 32 x 32 tiles
+// (pre_t: prefix sums of the merges' ceil(s / DC_TILE)^2 tiles; tiles past k exit).
+// FP64 multiply-adds at two per clock and SM bound it once every SM has tiles: 64 x 64
+// ones left most idle.  The same levels: 0.97 -> 0.51 ms.
+constexpr int DG_T = DC_TILE, DG_K = 16, DG_E = DG_T / 16;   // DG_E x DG_E results a thread
 
 __global__ void __launch_bounds__(256) dc_gemm_kernel(const DcMerge* __restrict__ ms, int nm,
                                                       const int* __restrict__ pre_t) {
@@ -400,11 +529,11 @@ __global__ void __launch_bounds__(256) dc_gemm_kernel(const DcMerge* __restrict_
   const int r0 = (t / ntc) * DG_T, c0 = (t % ntc) * DG_T;
   if (c0 >= k) return;
   const int tr = threadIdx.x & 15, tc = threadIdx.x >> 4;
-  double acc[4][4];
+  double acc[DG_E][DG_E];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < DG_E; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < DG_E; ++j) acc[i][j] = 0.0;
   for (int k0 = 0; k0 < k; k0 += DG_K) {
     for (int e = threadIdx.x; e < DG_T * DG_K; e += blockDim.x) {
       const int rr = e % DG_T, kk = e / DG_T;
@@ -419,25 +548,25 @@ __global__ void __launch_bounds__(256) dc_gemm_kernel(const DcMerge* __restrict_
     __syncthreads();
 #pragma unroll 4
     for (int kk = 0; kk < DG_K; ++kk) {
-      double a[4], b[4];
+      double a[DG_E], b[DG_E];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][tr + 16 * i];
+      for (int i = 0; i < DG_E; ++i) a[i] = As[kk][tr + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tc + 16 * j];
+      for (int j = 0; j < DG_E; ++j) b[j] = Bs[kk][tc + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < DG_E; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < DG_E; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < DG_E; ++j) {
     const int c = c0 + tc + 16 * j;
     if (c >= k) continue;
     double* zc = m.Z + int64_t(o + m.ndp[c]) * n + o;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < DG_E; ++i) {
       const int r = r0 + tr + 16 * i;
       if (r < s) zc[r] = acc[i][j];
     }
@@ -482,8 +611,8 @@ void launch_dc_merges(const DcMerge* m, int nmerge, const int* pre_s, int total,
   if (nmerge <= 0) return;
   dc_prep_kernel<<<unsigned(nmerge), DC_PREP_THREADS, 0, st>>>(m);
   dc_secular_kernel<<<unsigned((total + 7) / 8), 256, 0, st>>>(m, nmerge, pre_s);
-  dc_zhat_kernel<<<unsigned((total + 255) / 256), 256, 0, st>>>(m, nmerge, pre_s);
-  dc_ucol_kernel<<<unsigned((total + 255) / 256), 256, 0, st>>>(m, nmerge, pre_s);
+  dc_zhat_kernel<<<unsigned((total + 7) / 8), 256, 0, st>>>(m, nmerge, pre_s);
+  dc_ucol_kernel<<<unsigned((total + 7) / 8), 256, 0, st>>>(m, nmerge, pre_s);
   dc_qp_kernel<<<unsigned((total + 255) / 256), 256, 0, st>>>(m, nmerge, pre_s);
   dc_gemm_kernel<<<unsigned(ttotal), 256, 0, st>>>(m, nmerge, pre_t);
   dc_finish_kernel<<<unsigned(total), 128, 0, st>>>(m, nmerge, pre_s);
