@@ -271,7 +271,6 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
   std::vector<Tile> tiles;
   std::vector<int64_t> goct(gorder.size(), 0);
   double total = 0;
-  int64_t chunks = 0;
   for (size_t gi = 0; gi < gorder.size(); ++gi) {
     const size_t g = size_t(gorder[gi]);
     const int m0 = gpos[g], m1 = m0 + gcount[g];
@@ -305,13 +304,9 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
         const int nt = std::min(tn, cols - n0);
         tiles.push_back(Tile{int(gi), pos, last - pos + 1, int(r0), rows, n0, nt});
         total += part_cost(rows, nt, oct);
-        chunks += (oct + F64_CHUNK - 1) / F64_CHUNK;
       }
     }
   }
-  // sums are cut at whole chunks, a small launch's at thirds of them (its time is one
-  // unit's latency: a chunk is twelve stages in a row)
-  const int gran = chunks < 4 * int64_t(nsm) ? F64_CHUNK / 3 : F64_CHUNK;
   const double target = total / (4.0 * std::max(1, nsm));
   std::vector<F64Unit> units;
   std::vector<int> keys;
@@ -322,8 +317,8 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     const size_t g = size_t(gorder[size_t(t.g)]);
     const int m0 = gpos[g], i0 = member[size_t(m0)];
     const int cs = f0[size_t(i0)], nseg = f0[size_t(i0) + 1] - cs;
-    const int64_t oct = goct[size_t(t.g)], nch = (oct + gran - 1) / gran;
-    const double cc = (part_cost(t.rows, t.nt, F64_CHUNK) - 3000.0) * gran / F64_CHUNK;
+    const int64_t oct = goct[size_t(t.g)], nch = (oct + F64_CHUNK - 1) / F64_CHUNK;
+    const double cc = part_cost(t.rows, t.nt, F64_CHUNK) - 3000.0;
     const int64_t per = std::max<int64_t>(1, std::min<int64_t>(nch, int64_t(std::max(1.0, (target - 3000.0) / cc))));
     const int64_t parts = nch ? (nch + per - 1) / per : 1;
     F64Unit u{};
@@ -345,11 +340,11 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     u.noct = int(oct);
     if (want_tiles) out.tiles.push_back(u);
     for (int64_t q = 0; q < parts; ++q) {
-      // whole pieces of gran octets, spread evenly
+      // whole chunks, spread evenly
       const int64_t c0 = nch * q / parts, c1 = nch * (q + 1) / parts;
       u.sg = sg;
       u.k0 = k0;
-      u.noct = int(std::min<int64_t>(c1 * gran, oct) - c0 * gran);
+      u.noct = int(std::min<int64_t>(c1 * F64_CHUNK, oct) - c0 * F64_CHUNK);
       if (parts > 1) {
         u.part = out.npart;
         out.npart += int64_t(F64_TM) * n16;
