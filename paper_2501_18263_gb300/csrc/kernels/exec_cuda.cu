@@ -147,8 +147,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // one CTA per (range of elements, right-hand vector, group of MDOT_GRP vectors); every
 // product is summed over its threads and warps in the same order however the vectors
 // are grouped.  A group per CTA, not all vectors: with n in the thousands a launch had
-// two to four CTAs, each bound by the FP64 sums of 32 vectors (32 us at n = 4900,
-// m = 24; 6 us in groups of four)
+// two to four CTAs, each bound by the FP64 sums of 32 vectors (53 us a launch at
+// n = 15900 and m up to 24, 10 us in groups of four)
 constexpr int MDOT_GRP = 4;
 
 __global__ void __launch_bounds__(256) mdot_partial(const double* __restrict__ V, int64_t ldv, int m,
@@ -399,8 +399,12 @@ __device__ __forceinline__ int syev_find(const int* pre, int nj, int x) {
 //   -= v_r w + w_r v, stored, and its product with v' taken in the same breath;
 //   p is exchanged through global scratch (two buffers in turn: a CTA may be a pass
 //   ahead of one that still reads), w' = p - (tau / 2) (p . v') v'.
-// A column of order about 300 takes 10 us of which 3 are FP64 arithmetic (eight CTAs);
-// the two-pass form took 19.
+// Rows go to CTAs in turn, so that a short trailing block keeps all of them busy.
+// Bound by the latencies of a column (two sums over the CTA, a root and two quotients,
+// the barrier) and, for the first columns, the FP64 multiply-adds of the pass.  The 69
+// density matrices of a bond of L = 24, D = 1024 (orders up to 352): 6.5 ms with rows in
+// blocks of 32 per CTA and zeros summed by idle warps, 4.8 without the zeros, 4.1 now;
+// the two-pass form (clusters from order 256) took 13.0.
 __device__ __forceinline__ uint32_t syev_cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -469,7 +473,7 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
     double* A22 = A + int64_t(k + 1) * n + k + 1;
     double* pb = jb.pb + par * n;
     par ^= 1;
-    for (int r = rank * nw + wid; r < m; r += CS * nw) {
+    for (int r = wid * CS + rank; r < m; r += CS * nw) {
       double* a = A22 + int64_t(r) * n;
       const double vr = vs[r + 1], wr = ws[r + 1];
       double acc = 0.0;
@@ -512,9 +516,11 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
   }
 }
 
-// step 2: one warp per column of Q (pre: prefix sums of the matrices' n)
+// step 2: one warp per column of Q (pre: prefix sums of the matrices' n).  Column j is a
+// chain of j reflectors; neighbours go to different CTAs, so that the long chains of a
+// large matrix do not share an SM's FP64 pipes (same matrices: 0.99 -> 0.71 ms)
 __global__ void __launch_bounds__(256) syev_qform_kernel(const SyevJob* jobs, const int* pre, int nj) {
-  const int gw = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  const int gw = int((threadIdx.x >> 5) * gridDim.x + blockIdx.x), lane = threadIdx.x & 31;
   if (gw >= pre[nj]) return;
   const int b = syev_find(pre, nj, gw);
   const SyevJob jb = jobs[b];
@@ -1232,11 +1238,12 @@ class CudaExec : public Exec {
       jb.n = int(m);
       jb.pad = 0;
     }
-    // 1. the reduction: a cluster of SYEV_CLUSTER CTAs for each matrix of order >= 80
+    // 1. the reduction: a cluster of SYEV_CLUSTER CTAs for each matrix of order >= 64
     // (largest first), one CTA for each smaller one, whose arithmetic one SM does in the
-    // time a cluster takes for its barriers; 2. Q
+    // time a cluster takes for its barriers (the batch of syev_tridiag_kernel: 8.6 ms in
+    // all with the line at 48 or 64, 8.8 at 80, 9.2 at 112, 9.8 at 160); 2. Q
     std::vector<int> small, big;
-    for (int j = 0; j < nj; ++j) (n[j] >= 80 ? big : small).push_back(j);
+    for (int j = 0; j < nj; ++j) (n[j] >= 64 ? big : small).push_back(j);
     std::stable_sort(big.begin(), big.end(), [&](int a, int b) { return n[size_t(a)] > n[size_t(b)]; });
     SyevJob* dj = upload(jobs);
     int* dpn = upload(pre_n);

@@ -8,14 +8,15 @@
 // cheap beside it: one output per lane, a warp per 8 x 4 piece (any ragged tile is cut
 // with little waste), operands straight from the L1, the next eight k of both operands
 // loaded while the last eight are multiplied.  Measured: FP64 sigma of L = 32, D = 512
-// 53 ms (34 ms at 2 multiply-adds per clock and SM), of L = 16, D = 128 2.3 ms against
+// 50 ms (34 ms at 2 multiply-adds per clock and SM), of L = 16, D = 128 1.2 ms against
 // 203.8 and 10.6 ms for 64 x 64 tiles, whose warps idled on ragged edges and whose few
 // tiles left SMs without work; results are bit-identical to those tiles'.
 //
 // Long sums (F64_LONG octets and more) have few pieces and segments of a handful of k,
 // whose addresses take a warp longer than their multiply-adds: there each piece has two
 // warps, one that copies the operands of 16 k at a time, packed over segment borders,
-// into shared memory (cp.async), and one that only multiplies.
+// into shared memory (cp.async), and one that only multiplies (L = 16, D = 128: 1.8 ms
+// with one warp for both).
 #include "../exec_errors.h"
 #include "f64_tc.h"
 #include "tc.cuh"

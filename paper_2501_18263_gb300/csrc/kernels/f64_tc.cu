@@ -33,8 +33,8 @@
 // Tiles of at most 32 columns use half of TMEM and are double-buffered.
 //
 // Measured (FP64 sigma at the centre bond of L = 32, D = 512, 20.5 G multiply-adds in
-// ragged blocks of 1 to 140 rows): 14.0 ms, against 203.8 ms for 64 x 64 tiles of FP64
-// multiply-adds without stacking or a split of long sums, and 53 ms for the plain pieces
+// ragged blocks of 1 to 140 rows): 13.5 ms, against 203.8 ms for 64 x 64 tiles of FP64
+// multiply-adds without stacking or a split of long sums, and 50 ms for the plain pieces
 // of f64_plain.cu; relative error against 64 bits 6e-16 (plain: 1e-15) at L = 8, D = 64.
 #include <cuda_fp16.h>
 

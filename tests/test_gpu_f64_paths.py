@@ -51,7 +51,7 @@ def test_sigma_matches_the_oracle_and_scales_exactly(L, na, nb, D, bond):
     d.close()
 
 
-@pytest.mark.parametrize("orders", [(78, 79, 80, 81), (82, 87, 88, 89, 96), (127, 128, 129, 255, 256, 257)])
+@pytest.mark.parametrize("orders", [(62, 63, 64, 65), (78, 79, 80, 81, 82, 87, 88, 89, 96), (127, 128, 129, 255, 256, 257)])
 def test_eigensolver_around_the_cluster_threshold(orders):
     t, v = I.synthetic_integrals(2, 5)
     d = B.Dmrg(t, v, 1, 1, D=4, stream=stream())
