@@ -282,9 +282,8 @@ def main():
     pk, pk_kind = peaks()
     if prec == B.PREC_FP64:
         key = "gemm_f64"
-        mhz = pk.get("sm_max_mhz", 2070.0)
-        peak = 152 * 2 * 2 * mhz * 1e6 / 1e12   # 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x max clock
-        bound, unit, peak_kind = "alu", "TFLOP/s", "derived (152 SM x 2 DFMA/clk x 2 flop x sm_max_mhz)"
+        peak = pk["bf16_tflops"] / 36   # an FP64 multiply-add is 36 exact 16-bit digit products
+        bound, unit, peak_kind = "tensor", "TFLOP/s", f"{pk_kind} / 36 digit products"
     else:
         key = "gemm_bf16x"
         peak = pk["bf16_tflops"]

@@ -76,8 +76,7 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
                            int what = F64_UNITS | F64_TILES);
 
 // true for a launch that is faster in plain multiply-adds: a digit unit's latency (fill
-// the pipeline, one chunk, drain: about 12 us) is longer than what little there is to
-// compute.  The work is counted as the plain kernel pays for it, pieces of 8 x 4 and
+// the pipeline, one chunk, drain) is longer than what little there is to compute.  The work is counted as the plain kernel pays for it, pieces of 8 x 4 and
 // whole octets.  Sigma at L = 10, D = 100 / L = 6, D = 16 / L = 18, D = 24, one path
 // only -> this rule: 294 -> 272, 99 -> 76, 248 -> 239 us; any line between 1.5e6 and
 // 8e6 gives these times, with k counted without the octets' padding 1e6 is already too
