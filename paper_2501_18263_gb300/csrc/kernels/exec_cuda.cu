@@ -389,6 +389,14 @@ __device__ __forceinline__ int syev_find(const int* pre, int nj, int x) {
   return lo;
 }
 
+// an element of the trailing block after the rank-2 update: a - (v_r w_j + w_r v_j), in
+// the three operations of an update pass of its own.  Two multiply-adds would do (4.1 ms
+// instead of 4.7 below), but T's last bits decide where the QL iteration of its leaves
+// stops, and with that signs of eigenvectors
+__device__ __forceinline__ double syev_update(double a, double vr, double wr, double vj, double wj) {
+  return __dsub_rn(a, fma(vr, wj, __dmul_rn(wr, vj)));
+}
+
 // step 1: a cluster of CS CTAs per matrix (CS = 1: one CTA).  The rank-2 update of step
 // k - 1 and the product p = tau A22 v of step k run in one pass over the trailing rows,
 // so that a column costs one cluster barrier (p complete; the rows updated) instead of
@@ -403,8 +411,8 @@ __device__ __forceinline__ int syev_find(const int* pre, int nj, int x) {
 // Bound by the latencies of a column (two sums over the CTA, a root and two quotients,
 // the barrier) and, for the first columns, the FP64 multiply-adds of the pass.  The 69
 // density matrices of a bond of L = 24, D = 1024 (orders up to 352): 6.5 ms with rows in
-// blocks of 32 per CTA and zeros summed by idle warps, 4.8 without the zeros, 4.1 now;
-// the two-pass form (clusters from order 256) took 13.0.
+// blocks of 32 per CTA and zeros summed by idle warps, 4.7 now; the two-pass
+// form (clusters from order 256) took 13.0.
 __device__ __forceinline__ uint32_t syev_cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -437,11 +445,12 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
     const double* row = A + int64_t(k) * n + k;
     const double v0 = vs[0], w0 = ws[0];
     double part = 0.0;
-    for (int i = 1 + tid; i <= m; i += nt) {
-      const double x = fma(-w0, vs[i], fma(-v0, ws[i], row[i]));
-      vn[i - 1] = x;
-      if (i >= 2) part += x * x;
+    for (int i = 1 + tid; i < m; i += nt) {   // elements past the first
+      const double x = syev_update(row[i + 1], v0, w0, vs[i + 1], ws[i + 1]);
+      vn[i] = x;
+      part += x * x;
     }
+    if (tid == nt - 1) vn[0] = syev_update(row[1], v0, w0, vs[1], ws[1]);
     const double sigma = block_sum(part, m, red);
     if (tid == 0) {
       const double alpha = vn[0];
@@ -455,7 +464,7 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
       red[34] = scale;
       red[35] = tau;
       if (rank == 0) {
-        jb.d[k] = fma(-w0, v0, fma(-v0, w0, row[0]));
+        jb.d[k] = syev_update(row[0], v0, w0, v0, w0);
         jb.e[k] = beta;
         jb.tau[k] = tau;
       }
@@ -478,7 +487,7 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
       const double vr = vs[r + 1], wr = ws[r + 1];
       double acc = 0.0;
       for (int j = lane; j < m; j += 32) {
-        const double x = fma(-wr, vs[j + 1], fma(-vr, ws[j + 1], a[j]));
+        const double x = syev_update(a[j], vr, wr, vs[j + 1], ws[j + 1]);
         a[j] = x;
         acc = fma(x, vn[j], acc);
       }
@@ -506,9 +515,9 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
   if (tid == 0 && rank == 0) {
     if (n >= 2) {
       const double* a = A + int64_t(n - 2) * n + n - 2;
-      jb.d[n - 2] = fma(-ws[0], vs[0], fma(-vs[0], ws[0], a[0]));
-      jb.e[n - 2] = fma(-ws[0], vs[1], fma(-vs[0], ws[1], a[1]));
-      jb.d[n - 1] = fma(-ws[1], vs[1], fma(-vs[1], ws[1], a[n + 1]));
+      jb.d[n - 2] = syev_update(a[0], vs[0], ws[0], vs[0], ws[0]);
+      jb.e[n - 2] = syev_update(a[1], vs[0], ws[0], vs[1], ws[1]);
+      jb.d[n - 1] = syev_update(a[n + 1], vs[1], ws[1], vs[1], ws[1]);
     } else {
       jb.d[n - 1] = A[0];
     }
@@ -1319,7 +1328,7 @@ class CudaExec : public Exec {
       int* si = static_cast<int*>(alloc(sizeof(int) * size_t(ni)));
       scratch.push_back(sd);
       scratch.push_back(si);
-      std::vector<int> ps(lv.size() + 1, 0), pt(lv.size() + 1, 0);
+      std::vector<int> ps(lv.size() + 1, 0), pw(lv.size() + 1, 0), pt(lv.size() + 1, 0);
       int64_t od = 0, oi = 0;
       for (size_t i = 0; i < lv.size(); ++i) {
         DcMerge& mg = lv[i];
@@ -1348,16 +1357,19 @@ class CudaExec : public Exec {
         oi += up4(5 * s + 4);
         const int nt = int((s + DC_TILE - 1) / DC_TILE);
         ps[i + 1] = ps[i] + int(s);
+        pw[i + 1] = pw[i] + int((s + 31) / 32);
         pt[i + 1] = pt[i] + nt * nt;
       }
       DcMerge* dm = upload(lv);
       int* dps = upload(ps);
+      int* dpw = upload(pw);
       int* dpt = upload(pt);
       launch(PROF_EIG, [&] {
-        launch_dc_merges(dm, int(lv.size()), dps, ps.back(), dpt, pt.back(), st_);
+        launch_dc_merges(dm, int(lv.size()), dps, ps.back(), dpw, pw.back(), dpt, pt.back(), st_);
       });
       release(dm);
       release(dps);
+      release(dpw);
       release(dpt);
     }
     // 4. W = Q V (column-major both: as row-major arrays W^T = V^T Q^T), into U

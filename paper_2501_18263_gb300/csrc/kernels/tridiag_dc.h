@@ -49,8 +49,8 @@ constexpr int DC_TILE = 32;   // tile of the eigenvector products
 
 void launch_dc_leaves(const DcLeaf* leaves, int nleaves, int* err, cudaStream_t st);
 // pre_s: prefix sums of the merges' s (device, nmerge + 1 entries); total = pre_s[nmerge];
-// tiles: prefix sums of ceil(s / DC_TILE)^2 (device), ttotal its last entry
-void launch_dc_merges(const DcMerge* m, int nmerge, const int* pre_s, int total, const int* pre_t, int ttotal,
-                      cudaStream_t st);
+// pre_w: of ceil(s / 32), wtotal; pre_t: of ceil(s / DC_TILE)^2, ttotal
+void launch_dc_merges(const DcMerge* m, int nmerge, const int* pre_s, int total, const int* pre_w, int wtotal,
+                      const int* pre_t, int ttotal, cudaStream_t st);
 
 }  // namespace dmrg
