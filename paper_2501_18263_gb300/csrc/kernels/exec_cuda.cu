@@ -421,6 +421,7 @@ __device__ __forceinline__ uint32_t syev_cluster_rank() {
 
 __device__ __forceinline__ void syev_cluster_sync() {
   __threadfence();
+  __syncwarp();   // lane 0's store of a row's product diverges; the barrier is .aligned
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

@@ -678,6 +678,7 @@ __global__ void __maxnreg__(REGS)
           if (nOct > 0) {
             float a[8][4];
             bool bad = false;
+            __syncwarp();   // the stores of the columns before diverge; the load is .aligned
             tmem_ld8x4(tq + 256u * b0 + uint32_t(cb + hh), uint32_t(n16), a);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {

@@ -67,7 +67,8 @@ __device__ __forceinline__ int dc_find(const int* pre, int nj, int x) {
 
 // ---- leaves: one warp each, lane r holds row r of the leaf's eigenvectors in
 // shared memory; the lanes look for negligible couplings, run the QL recurrences of one
-// iteration (the rotations recorded by lane 0), then every lane applies them to its row.  More than 60 iterations for one eigenvalue: *err = 9.
+// iteration (the rotations recorded by lane 0), then every lane applies them to its row.
+// More than 60 iterations for one eigenvalue: *err = 9.
 //
 // Bound by the chain of dependent FP64 instructions, about 900 rotations of a hypot and
 // two quotients for 32 rows.  The leaves of the density matrices of one bond at L = 24,
