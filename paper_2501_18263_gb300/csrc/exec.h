@@ -147,8 +147,10 @@ class Exec {
   virtual void kron(const std::vector<KronGroup>& g, const std::vector<KronTask>& t) = 0;
   // grouped, segmented FP64 GEMM (one-shot upload).  plain: every element by FP64
   // multiply-adds in the order of its segments and k, so that its rounding does not
-  // depend on the launch; otherwise the executor may use its tensor-core form (error
-  // no larger, another rounding sequence)
+  // depend on the launch; otherwise the executor may use its tensor-core form: another
+  // rounding sequence, errors of the size of FP64 rounding relative to the row's largest
+  // element times the column's (normwise no larger), and within 2^-36 of every element's
+  // own terms (f64_digits.h), where multiply-adds are within k 2^-53
   virtual void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain = false) = 0;
   // persistent plans (uploaded once, replayed during Davidson); forms: what gemm_run may
   // be asked for (GEMM_ANY: plain = false, GEMM_PLAIN: plain = true, or both)

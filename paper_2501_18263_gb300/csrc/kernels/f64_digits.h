@@ -99,13 +99,25 @@ F64_HD void f64_combine(float a0, float a1, float a2, float a3, float a4, float 
   lo = uint32_t(t) << 8;
 }
 
+// A sum too small for its digits: |V| < 2^F64_WEAK, where a product of the row's and the
+// column's largest elements has |V| of 2^66 to 2^68.  V is off by at most 578 k + 2^14
+// (weights above 7: below 450 a product; elements cut at 2^-62 of the largest: below 128;
+// the sums of weights 6 and 7 in FP32), so a sum of terms that are each far below the
+// largest row element times the largest column element has lost bits that plain
+// multiply-adds keep.  Such sums are computed again, plainly; the others are within
+// 2^-36 of their own value and, as a rule (errors of either sign), within 2^-44.
+// lead: the leading zero bits of |V| as 96 bits.
+constexpr int F64_WEAK = 54;
+F64_HD bool f64_weak(int lead) { return lead >= 96 - F64_WEAK; }
+
 // The double nearest to (hi 2^32 + lo) 2^(ea + eb - 2112), its sign flipped when `flip`
 // (integer instructions only in the normal range: an FP64 one costs 16 times as much
 // here).
 //
 // f64_assemble_fast: without branches, so that several elements' chains interleave;
-// *bad is set where the result is not a normal number below 2^1023 or zero.
-F64_HD double f64_assemble_fast(int64_t hi, uint32_t c0, int ea, int eb, bool flip, bool* bad) {
+// *bad is set where the result is not a normal number below 2^1023 or zero; *lead: the
+// leading zero bits of |V|.
+F64_HD double f64_assemble_fast(int64_t hi, uint32_t c0, int ea, int eb, bool flip, bool* bad, int* lead = nullptr) {
   const bool neg = hi < 0;
   // |V| as three words
   const uint64_t m = neg ? ~uint64_t(hi) + (c0 == 0 ? 1 : 0) : uint64_t(hi);
@@ -119,7 +131,9 @@ F64_HD double f64_assemble_fast(int64_t hi, uint32_t c0, int ea, int eb, bool fl
   a = z2 ? b : a;
   b = z2 ? 0u : b;
   const int lz = f64_clz32(a);
-  const int E = ea + eb - 994 - (z1 ? 32 : 0) - (z2 ? 32 : 0) - lz;
+  const int zeros = (z1 ? 32 : 0) + (z2 ? 32 : 0) + lz;
+  if (lead) *lead = zeros;
+  const int E = ea + eb - 994 - zeros;
   // (w1:w0) 2^(E - 1086): the top bit of w1 set; 53 bits kept, rounded to nearest
   const uint32_t w1 = f64_shl(a, b, lz), w0 = f64_shl(b, c, lz);
   const uint64_t mant = ((uint64_t(w1 >> 11) << 32) | f64_shl(w1, w0, 21)) + ((w0 >> 10) & 1u);

@@ -6,11 +6,15 @@
 // (2012)): every row of A and every column of B is scaled by its largest exponent
 // over a chunk of K and written as eight signed 8-bit digits (f64_digits.h).  A digit
 // is exact in FP16, a product of two in FP32, and so are the sums over a chunk (at
-// most 192 k) of the digit products of equal weight, so that
+// most 192 k) of the digit products of equal weight (0 to 5; those of weights 6 and 7,
+// worth 2^-56 and less of the largest product, may round), so that
 //   acc[w] = sum_k sum_{i + j = w} dA_i dB_j,   w = 0 .. 7,
-// gives A B up to 2^-60 of the largest products; the 36 products per k replace one
-// FP64 multiply-add.  The accumulators are combined in integers, rounded once to FP64
-// and added over the chunks in FP64.  Rows or columns with an infinity or a NaN are
+// gives A B up to 2^-58 a k of the row's largest element times the column's (each up to
+// the power of two above it); the 36 products per k replace one FP64 multiply-add.  The
+// accumulators are combined in integers, rounded once to FP64 and added over the chunks
+// in FP64.  The error is normwise: an element 2^9 or more below its row's largest is held
+// in fewer than 53 bits.  Elements of C whose chunk sum comes out far below what its row
+// and column could give (f64_weak), and rows or columns with an infinity or a NaN, are
 // computed by plain FP64 multiply-adds.
 //
 // One tile: 128 rows (TMEM lanes) x up to 64 columns, eight accumulators of 64 TMEM
@@ -33,9 +37,11 @@
 // Tiles of at most 32 columns use half of TMEM and are double-buffered.
 //
 // Measured (FP64 sigma at the centre bond of L = 32, D = 512, 20.5 G multiply-adds in
-// ragged blocks of 1 to 140 rows): 13.5 ms, against 203.8 ms for 64 x 64 tiles of FP64
+// ragged blocks of 1 to 140 rows): 14.1 ms, against 203.8 ms for 64 x 64 tiles of FP64
 // multiply-adds without stacking or a split of long sums, and 50 ms for the plain pieces
 // of f64_plain.cu; relative error against 64 bits 6e-16 (plain: 1e-15) at L = 8, D = 64.
+// Small sums computed again cost 0.6 ms of it (about one element in 5000 of dense
+// operators; with the line of f64_weak at 2^52 13.9 ms, 2^56 14.9, 2^58 18.8, 2^60 31).
 #include <cuda_fp16.h>
 
 #include <atomic>
@@ -69,7 +75,7 @@ struct Slot {
   int first;           // first chunk of its unit (pos is written then)
   int ci;              // chunk of the unit
   int rows, n0, nt, cs, trans;
-  int unit, pad;
+  int pad[2];
   int64_t part;
   int2 oct[F64_CHUNK]; // segment; 16 x first k + length
   int s0[F64_TM];      // per row: its problem's first segment, its row there
@@ -158,26 +164,41 @@ __device__ __forceinline__ int locate(const F64Row* __restrict__ rows, int pos0,
   return pos;
 }
 
-// plain FP64 dot product over the octets [o0, o0 + no) of a unit (rows or columns
-// that hold an infinity or a NaN)
-__device__ __noinline__ double plain_dot(const F64Unit* __restrict__ u, const F64Ref* __restrict__ ra,
-                                         const F64Ref* __restrict__ rb, int m, int n, int o0, int no) {
+// one element's sum over the slot's octets by plain FP64 multiply-adds, a k per lane
+// (warp-collective, the sum on every lane): rows or columns that hold an infinity or a
+// NaN, and sums too small for their digits.  Twelve octets at a time, all their records
+// loaded before any element: it is bound by the two latencies
+__device__ __noinline__ double chunk_dot(const Slot* S, const F64Ref* __restrict__ ra, const F64Ref* __restrict__ rb,
+                                         int m, int n, int nOct) {
+  const int lane = threadIdx.x & 31, kl = lane & 7;
   double acc = 0.0;
-  int s = u->sg, k = u->k0, o = 0;
-  while (o < o0 + no) {
-    const F64Ref a = ra[s], b = rb[s];
-    const int K = a.kt >> 1;
-    for (; k < K && o < o0 + no; k += 8, ++o) {
-      if (o < o0) continue;
-      for (int q = k; q < min(K, k + 8); ++q) {
-        const double x = (a.kt & 1) ? a.p[int64_t(q) * a.ld + m] : a.p[int64_t(m) * a.ld + q];
-        const double y = (b.kt & 1) ? b.p[int64_t(q) * b.ld + n] : b.p[int64_t(n) * b.ld + q];
-        acc = fma(x, y, acc);
-      }
+#pragma unroll 1
+  for (int h = 0; h < nOct; h += 12) {
+    int2 e[3];
+    int4 fa[3], fb[3];
+    double x[3], y[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      e[q] = S->oct[h + 4 * q + (lane >> 3)];   // octets past the last have no k
+      fa[q] = __ldg(reinterpret_cast<const int4*>(ra + e[q].x));
+      fb[q] = __ldg(reinterpret_cast<const int4*>(rb + e[q].x));
     }
-    ++s;
-    k = 0;
+    auto at = [](const int4& f, int r, int k) {
+      const double* p = reinterpret_cast<const double*>((uint64_t(uint32_t(f.y)) << 32) | uint32_t(f.x));
+      return __ldg(p + ((f.w & 1) ? int64_t(k) * f.z + r : int64_t(r) * f.z + k));
+    };
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int k = (e[q].y >> 4) + kl;
+      const bool on = kl < (e[q].y & 15);
+      x[q] = on ? at(fa[q], m, k) : 0.0;
+      y[q] = on ? at(fb[q], n, k) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) acc = fma(x[q], y[q], acc);
   }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
   return acc;
 }
 
@@ -574,7 +595,6 @@ __global__ void __maxnreg__(REGS)
             S.nt = u->nt;
             S.cs = cs;
             S.trans = u->trans;
-            S.unit = ui;
             S.part = u->part;
           }
           __syncwarp();
@@ -643,6 +663,7 @@ __global__ void __maxnreg__(REGS)
       const bool wide = n16 > 32;
       const int b0 = wide ? 0 : tog;
       int ea = 1;
+      bool special = false;   // a row or column of the tile holds an infinity or a NaN
       if (nOct > 0) {
         if (!wide) tog ^= 1;
         if (!mbar_wait_warp(ex_full(sl), (chunk / SLOTS) & 1, abort_flag, err, 18) ||
@@ -651,33 +672,24 @@ __global__ void __maxnreg__(REGS)
         ++(b0 ? seen1 : seen0);
         fence_after();
         ea = rv ? max(S.expo[r] >> 20, 1) : 1;
+        special = __any_sync(0xffffffffu, ea == F64_SPECIAL ||
+                                              (lane < nt && (S.expo[F64_TM + lane] >> 20) == F64_SPECIAL) ||
+                                              (lane + 32 < nt && (S.expo[F64_TM + 32 + lane] >> 20) == F64_SPECIAL));
       }
       if (!direct) {
-        // row pointers for the staged stores; bit 0: add to C, bit 1: special row
-        ptrs[lane] = reinterpret_cast<uint64_t>(out) | (old ? 1u : 0u) | (ea == F64_SPECIAL ? 2u : 0u);
+        // row pointers for the staged stores; bit 0: add to C
+        ptrs[lane] = reinterpret_cast<uint64_t>(out) | (old ? 1u : 0u);
         __syncwarp();
       }
       // (a quarter without rows has nothing to do)
       for (int cb = half * (n16 >> 1); cb < (half + 1) * (n16 >> 1) && cb < nt && quarter * 32 < nrows; cb += 8) {
-        // a lane's column of the block, for the stores through shared memory
-        const bool colsp = nOct > 0 && (S.expo[F64_TM + min(cb + (lane & 7), nt - 1)] >> 20) == F64_SPECIAL;
-        if (__any_sync(0xffffffffu, ea == F64_SPECIAL || colsp)) {
-          // infinities or NaN: these elements apart, and left out below
-#pragma unroll 1
-          for (int c = cb; c < min(cb + 8, nt); ++c)
-            if (rv && (ea == F64_SPECIAL || (S.expo[F64_TM + c] >> 20) == F64_SPECIAL)) {
-              const double x = alpha * plain_dot(units + S.unit, rowref + s0, colref + S.cs, m, S.n0 + c,
-                                                 F64_CHUNK * S.ci, nOct);
-              double* p = out + (direct ? int64_t(c) * cstr : int64_t(c));
-              *p = old ? *p + x : x;
-            }
-        }
 #pragma unroll 1
         for (int hh = 0; hh < 8; hh += 4) {
           double v[4] = {0.0, 0.0, 0.0, 0.0};
           if (nOct > 0) {
             float a[8][4];
             bool bad = false;
+            uint32_t again = 0;   // elements that digits do not give (well enough)
             __syncwarp();   // the stores of the columns before diverge; the load is .aligned
             tmem_ld8x4(tq + 256u * b0 + uint32_t(cb + hh), uint32_t(n16), a);
 #pragma unroll
@@ -686,8 +698,11 @@ __global__ void __maxnreg__(REGS)
               int64_t hi;
               uint32_t lo;
               f64_combine(a[0][i], a[1][i], a[2][i], a[3][i], a[4][i], a[5][i], a[6][i], a[7][i], hi, lo);
-              v[i] = f64_assemble_fast(hi, lo, ea, max(S.expo[F64_TM + min(cb + hh + i, nt - 1)] >> 20, 1), flip, &bd);
+              int lead;
+              v[i] = f64_assemble_fast(hi, lo, ea, max(S.expo[F64_TM + min(cb + hh + i, nt - 1)] >> 20, 1), flip, &bd,
+                                       &lead);
               bad |= bd && rv;
+              again |= f64_weak(lead) ? 1u << i : 0u;
             }
             if (__any_sync(0xffffffffu, bad)) {   // results outside the normal range
 #pragma unroll
@@ -698,6 +713,28 @@ __global__ void __maxnreg__(REGS)
                 v[i] = assemble_any(hi, lo, ea, max(S.expo[F64_TM + min(cb + hh + i, nt - 1)] >> 20, 1), flip);
               }
             }
+            if (special || __any_sync(0xffffffffu, again != 0)) {
+              const int xa = rv ? S.expo[r] : 0;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {   // (a sum of nothing but zeros is one)
+                const int xb = S.expo[F64_TM + min(cb + hh + i, nt - 1)];
+                const bool sp = (xa >> 20) == F64_SPECIAL || (xb >> 20) == F64_SPECIAL;
+                const bool terms = (xa != 0 && xb != 0) || __double_as_longlong(v[i]) << 1 != 0;
+                if (!rv || cb + hh + i >= nt || !(sp || terms)) again &= ~(1u << i);
+                else if (sp) again |= 1u << i;
+              }
+              for (uint32_t left = __ballot_sync(0xffffffffu, again != 0); left; left &= left - 1) {
+                const int l = __ffs(int(left)) - 1;
+                const uint32_t todo = __shfl_sync(0xffffffffu, again, l);
+                const int ml = __shfl_sync(0xffffffffu, m, l), sl0 = __shfl_sync(0xffffffffu, s0, l);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  if (!(todo >> i & 1u)) continue;
+                  const double x = chunk_dot(&S, rowref + sl0, colref + S.cs, ml, S.n0 + cb + hh + i, nOct);
+                  if (lane == l) v[i] = flip ? -x : x;
+                }
+              }
+            }
           }
           if (any_other) {   // factors other than +-1 (warp-uniform)
             asm volatile("" ::: "memory");   // kept a branch: FP64 instructions are slow
@@ -705,7 +742,7 @@ __global__ void __maxnreg__(REGS)
             for (int i = 0; i < 4; ++i) v[i] *= flip ? 1.0 : alpha;
           }
           if (direct) {
-            if (rv && ea != F64_SPECIAL) {
+            if (rv) {
               double* p = out + int64_t(cb + hh) * cstr;
               if (any_old) {
                 double c[4];
@@ -716,7 +753,7 @@ __global__ void __maxnreg__(REGS)
               }
 #pragma unroll
               for (int i = 0; i < 4; ++i)
-                if (cb + hh + i < nt && (nOct == 0 || (S.expo[F64_TM + cb + hh + i] >> 20) != F64_SPECIAL)) p[i * cstr] = v[i];
+                if (cb + hh + i < nt) p[i * cstr] = v[i];
             }
           } else {
 #pragma unroll
@@ -734,8 +771,8 @@ __global__ void __maxnreg__(REGS)
             const int sr = 4 * it + (lane >> 3);
             const uint64_t po = ptrs[sr];
             v[it] = stg[sr * STG_LD + cc];
-            const bool on = quarter * 32 + sr < nrows && cb + cc < nt && !(po & 2) && !colsp;
-            p[it] = on ? reinterpret_cast<double*>(po & ~uint64_t(3)) + cb + cc : nullptr;
+            const bool on = quarter * 32 + sr < nrows && cb + cc < nt;
+            p[it] = on ? reinterpret_cast<double*>(po & ~uint64_t(1)) + cb + cc : nullptr;
             if (any_old && on && (po & 1)) v[it] += *p[it];
           }
 #pragma unroll
