@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <stdexcept>
 
 namespace dmrg {
 
@@ -82,6 +83,11 @@ bool f64_small(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) {
     if (mac > F64_SMALL_MAC) return false;
   }
   return true;
+}
+
+bool f64_run_plain(int forms, bool small, bool plain) {
+  if (!(forms & (plain ? GEMM_PLAIN : GEMM_ANY))) throw std::logic_error("gemm_run: the plan was built without this form");
+  return plain || small;
 }
 
 F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int nsm, int what) {

@@ -86,4 +86,9 @@ constexpr double F64_SMALL_MAC = 3e6;
 constexpr int64_t F64_SMALL_K = 512;
 bool f64_small(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s);
 
+// whether a run of a plan built for `forms` (GEMM_ANY, GEMM_PLAIN) goes to the plain
+// kernel; throws std::logic_error when the form asked for is not among them (the plan
+// may hold no work in it, and C would keep its old contents)
+bool f64_run_plain(int forms, bool small, bool plain);
+
 }  // namespace dmrg

@@ -841,6 +841,7 @@ class CudaExec : public Exec {
     int* next = nullptr;
     double* part = nullptr;
     int nunits = 0, nreds = 0, nlong = 0, plong = 0, ntiles = 0, npieces = 0;
+    int forms = 0;          // GEMM_ANY, GEMM_PLAIN
     bool small = false;     // plain in any case
     bool live = false;
   };
@@ -850,6 +851,7 @@ class CudaExec : public Exec {
     const F64PlanHost h = f64_build_plan(
         p, s, nsm_, (forms & GEMM_ANY && !small ? F64_UNITS : 0) | (forms & GEMM_PLAIN || small ? F64_TILES : 0));
     Plan pl;
+    pl.forms = forms;
     pl.small = small;
     pl.nunits = int(h.units.size());
     pl.nreds = int(h.reds.size());
@@ -903,8 +905,8 @@ class CudaExec : public Exec {
   }
   void gemm_run(int id, bool plain) override {
     Plan& pl = plans_.at(id);
-    plain = plain || pl.small;
-    if (!(plain ? pl.ntiles : pl.nunits)) return;
+    plain = f64_run_plain(pl.forms, pl.small, plain);
+    if (!(plain ? pl.ntiles : pl.nunits)) return;   // no outputs
     launch(PROF_GEMM, [&] {
       if (plain) {
         launch_gemm_f64_plain(pl.tiles, pl.pieces, pl.nlong, pl.plong, pl.ntiles, pl.npieces, pl.rows, pl.rowref,

@@ -1,9 +1,11 @@
-// Host forms of the FP64 digit kernel's rules (csrc/kernels/f64_digits.h), for
-// test_f64_rules.py.
+// Host forms of the FP64 digit kernel's rules (csrc/kernels/f64_digits.h,
+// csrc/core/f64_plan.h), for test_f64_rules.py.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <stdexcept>
 
+#include "core/f64_plan.h"
 #include "kernels/f64_digits.h"
 
 using namespace dmrg;
@@ -41,4 +43,13 @@ extern "C" int f64_chunk(const double* a, const double* b, int K, double* out) {
   *out = 0.0;
   for (int k = 0; k < K; ++k) *out = std::fma(a[k], b[k], *out);
   return 1;
+}
+
+// 1 plain, 0 digits, -1 refused
+extern "C" int f64_route(int forms, int small, int plain) {
+  try {
+    return f64_run_plain(forms, small, plain) ? 1 : 0;
+  } catch (const std::logic_error&) {
+    return -1;
+  }
 }

@@ -19,8 +19,9 @@ CSRC = os.path.join(os.path.dirname(HERE), "paper_2501_18263_gb300", "csrc")
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("f64") / "rules.so")
-    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC,
-                    os.path.join(HERE, "f64_rules_emulate.cpp"), "-o", so], check=True)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-pthread", "-I" + CSRC,
+                    os.path.join(HERE, "f64_rules_emulate.cpp"), os.path.join(CSRC, "core", "f64_plan.cpp"), "-o", so],
+                   check=True)
     return ctypes.CDLL(so)
 
 
@@ -58,3 +59,13 @@ def test_few_ordinary_sums_are_computed_again(lib, K):
     rng = np.random.default_rng(K)
     again = [_chunk(lib, rng.standard_normal(K), rng.standard_normal(K))[0] for _ in range(4000)]
     assert np.mean(again) < 2e-3
+
+
+ANY, PLAIN = 1, 2
+
+
+@pytest.mark.parametrize("forms, small, plain, route", [
+    (ANY, 0, 0, 0), (ANY, 1, 0, 1), (PLAIN, 0, 1, 1), (PLAIN, 1, 1, 1), (ANY | PLAIN, 0, 0, 0), (ANY | PLAIN, 0, 1, 1),
+    (ANY | PLAIN, 1, 0, 1), (ANY, 0, 1, -1), (ANY, 1, 1, -1), (PLAIN, 0, 0, -1), (PLAIN, 1, 0, -1), (0, 0, 0, -1)])
+def test_a_plan_runs_only_in_a_form_it_was_built_for(lib, forms, small, plain, route):
+    assert lib.f64_route(forms, small, plain) == route
