@@ -13,6 +13,7 @@
 #include <functional>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -839,12 +840,30 @@ class CudaExec : public Exec {
     F64Unit* tiles = nullptr;
     int* pieces = nullptr;
     int* next = nullptr;
-    double* part = nullptr;
+    std::shared_ptr<double> part;
     int nunits = 0, nreds = 0, nlong = 0, plong = 0, ntiles = 0, npieces = 0;
     int forms = 0;          // GEMM_ANY, GEMM_PLAIN
     bool small = false;     // plain in any case
     bool live = false;
   };
+
+  // Partial sums of split products, n doubles: they live from a plan's kernel to its
+  // reduction, and a handle's plans run one after another on its stream, so that they
+  // share one buffer (a plan each: 1.2 GB for the 778 plans of L = 24, D = 512 under a cap
+  // of 64 MB, against 8 MB of the largest).  A plan that needs more gets a new one, twice
+  // as large or more; the old one goes with the last plan that holds it (a bond's graphs
+  // are freed before its plans).
+  std::shared_ptr<double> partial_sums(size_t n) {
+    std::shared_ptr<double> p = sums_.lock();
+    if (p && sums_n_ >= n) return p;
+    size_t cap = size_t(1) << 17;
+    while (cap < n) cap *= 2;
+    const cudaStream_t st = st_;
+    p.reset(static_cast<double*>(alloc(sizeof(double) * cap)), [st](double* d) { cudaFreeAsync(d, st); });
+    sums_ = p;
+    sums_n_ = cap;
+    return p;
+  }
 
   int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int forms) override {
     const bool small = f64_small(p, s);
@@ -853,6 +872,7 @@ class CudaExec : public Exec {
     Plan pl;
     pl.forms = forms;
     pl.small = small;
+    if (h.npart) pl.part = partial_sums(size_t(h.npart));
     pl.nunits = int(h.units.size());
     pl.nreds = int(h.reds.size());
     pl.ntiles = int(h.tiles.size());
@@ -893,7 +913,6 @@ class CudaExec : public Exec {
     pl.reds = reinterpret_cast<F64Red*>(d + off[4]);
     pl.tiles = reinterpret_cast<F64Unit*>(d + off[5]);
     pl.pieces = reinterpret_cast<int*>(d + off[6]);
-    if (h.npart) pl.part = static_cast<double*>(alloc(sizeof(double) * size_t(h.npart)));
     pl.live = true;
     for (size_t i = 0; i < plans_.size(); ++i)
       if (!plans_[i].live) {
@@ -913,14 +932,14 @@ class CudaExec : public Exec {
                               pl.colref, err_, st_);
         return;
       }
-      launch_gemm_f64_tc(pl.units, pl.nunits, pl.rows, pl.rowref, pl.colref, pl.part, pl.reds, pl.nreds, pl.next, err_, nsm_,
+      launch_gemm_f64_tc(pl.units, pl.nunits, pl.rows, pl.rowref, pl.colref, pl.part.get(), pl.reds, pl.nreds, pl.next, err_, nsm_,
                          st_);
     });
   }
   void free_plan_mem(Plan& p) {
     if (!p.live) return;
     cudaFreeAsync(p.mem, st_);
-    if (p.part) cudaFreeAsync(p.part, st_);
+    p.part.reset();
     p.live = false;
   }
   void plan_free(int id) override { free_plan_mem(plans_.at(id)); }
@@ -1420,6 +1439,8 @@ class CudaExec : public Exec {
   std::vector<cudaGraphExec_t> graphs_;
   double* part_ = nullptr;
   std::vector<Plan> plans_;
+  std::weak_ptr<double> sums_;
+  size_t sums_n_ = 0;
 };
 
 Exec* make_cuda_exec(void* stream, int precision_mode) { return new CudaExec(stream, precision_mode); }
