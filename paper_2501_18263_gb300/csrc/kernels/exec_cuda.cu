@@ -21,6 +21,7 @@
 #include "../exec_errors.h"
 #include "f64_tc.h"
 #include "mixed.h"
+#include "syev_shared.h"
 #include "tridiag_dc.h"
 
 namespace dmrg {
@@ -351,6 +352,7 @@ struct SyevJob {
   double* Zc;     // n x n, column-major (Zc[c * n + r]): Q
   double* U;      // n x n: reflector k in row k (u_k[k + 1] = 1), then W = Q V (column-major)
   double* pb;     // 2 n: p = tau A22 v exchanged between the CTAs of a cluster
+  double* far;    // SYEV_CLUSTER n: a vector for each CTA (orders past syev_shared's line)
   int* perm;      // n: sorted position of eigenvalue i
   int n, pad;
 };
@@ -426,7 +428,7 @@ __device__ __forceinline__ void syev_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <int CS>
+template <int CS, bool FAR>
 __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJob* jobs, const int* sel, int maxn) {
   const int rank = CS > 1 ? int(syev_cluster_rank()) : 0;
   const SyevJob jb = jobs[sel[blockIdx.x / CS]];
@@ -435,8 +437,9 @@ __global__ void __launch_bounds__(SYEV_THREADS) syev_tridiag_kernel(const SyevJo
   extern __shared__ double sm[];
   double* vs = sm;             // v and w of the step before (element i: row k + i), zero at first
   double* ws = vs + maxn;
-  double* vn = ws + maxn;      // row k, then the reflector (element i: row k + 1 + i)
-  double* red = vn + maxn;     // 40 doubles: reductions and scalars
+  // row k, then the reflector (element i: row k + 1 + i)
+  double* vn = FAR ? jb.far + int64_t(rank) * n : ws + maxn;
+  double* red = ws + (FAR ? 1 : 2) * maxn;   // 40 doubles: reductions and scalars
   double* A = jb.A;
   for (int i = tid; i < n; i += nt) vs[i] = ws[i] = 0.0;
   bool pending = false;
@@ -1226,27 +1229,26 @@ class CudaExec : public Exec {
             const std::vector<int>& n) override {
     if (A.empty()) return;
     const int nj = int(A.size());
-    // per matrix: d, e, tau, pb (5n), Zc, U (2 n^2) doubles; perm (n) ints; every
+    // per matrix: d, e, tau, pb (5n), Zc, U (2 n^2), far doubles; perm (n) ints; every
     // part 16-byte aligned
     auto up2 = [](int64_t x) { return (x + 1) & ~int64_t(1); };
     auto up4 = [](int64_t x) { return (x + 3) & ~int64_t(3); };
     std::vector<int64_t> doff(nj), ioff(nj);
     std::vector<int> pre_n(nj + 1, 0);
     int64_t dtot = 0, itot = 0;
-    int maxn = 2;
+    const SyevShared sh = syev_shared(*std::max_element(n.begin(), n.end()));
+    const int maxn = sh.len;
     for (int j = 0; j < nj; ++j) {
       const int64_t m = n[j];
       if (m <= 0) throw std::runtime_error("syev: empty matrix");
       if (m > 32767) throw std::runtime_error("syev: matrix order above 32767");
       doff[j] = dtot;
-      dtot += up2(5 * m) + 2 * up2(m * m);
+      dtot += up2(5 * m) + 2 * up2(m * m) + (sh.far ? up2(SYEV_CLUSTER * m) : 0);
       ioff[j] = itot;
       itot += up4(m);
       pre_n[j + 1] = pre_n[j] + int(m);
-      maxn = std::max(maxn, int(m) + 2);
     }
-    const size_t smem1 = sizeof(double) * (3 * size_t(maxn) + 40);
-    if (smem1 > 227 * 1024) throw std::runtime_error("syev: matrix too large for the shared-memory workspace");
+    const size_t smem1 = sh.bytes;
     double* dw = static_cast<double*>(alloc(sizeof(double) * size_t(dtot)));
     int* iw = static_cast<int*>(alloc(sizeof(int) * size_t(itot)));
     std::vector<SyevJob> jobs(nj);
@@ -1265,6 +1267,7 @@ class CudaExec : public Exec {
       jb.Zc = p;
       p += up2(m * m);
       jb.U = p;
+      jb.far = p + up2(m * m);
       jb.perm = iw + ioff[j];
       jb.n = int(m);
       jb.pad = 0;
@@ -1280,15 +1283,16 @@ class CudaExec : public Exec {
     int* dpn = upload(pre_n);
     int* dsmall = upload(small);
     int* dbig = upload(big);
+    const auto one = sh.far ? syev_tridiag_kernel<1, true> : syev_tridiag_kernel<1, false>;
+    const auto many = sh.far ? syev_tridiag_kernel<SYEV_CLUSTER, true> : syev_tridiag_kernel<SYEV_CLUSTER, false>;
     if (smem1 > 48 * 1024) {
-      CK(cudaFuncSetAttribute(syev_tridiag_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem1)));
-      CK(cudaFuncSetAttribute(syev_tridiag_kernel<SYEV_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(smem1)));
+      CK(cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem1)));
+      CK(cudaFuncSetAttribute(many, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem1)));
     }
     const int ncol = pre_n[nj];
     if (!small.empty())
       launch(PROF_EIG, [&] {
-        syev_tridiag_kernel<1><<<unsigned(small.size()), SYEV_THREADS, smem1, st_>>>(dj, dsmall, maxn);
+        one<<<unsigned(small.size()), SYEV_THREADS, smem1, st_>>>(dj, dsmall, maxn);
       });
     if (!big.empty())
       launch(PROF_EIG, [&] {
@@ -1304,8 +1308,7 @@ class CudaExec : public Exec {
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        CK(cudaLaunchKernelEx(&cfg, syev_tridiag_kernel<SYEV_CLUSTER>, static_cast<const SyevJob*>(dj),
-                              static_cast<const int*>(dbig), maxn));
+        CK(cudaLaunchKernelEx(&cfg, many, static_cast<const SyevJob*>(dj), static_cast<const int*>(dbig), maxn));
       });
     launch(PROF_EIG, [&] { syev_qform_kernel<<<unsigned((ncol + 7) / 8), 256, 0, st_>>>(dj, dpn, nj); });
     // 3. T = V diag(d) V^T by divide and conquer: the blocks are halved until they
