@@ -51,6 +51,7 @@ inline int up16(int x) { return (x + 15) & ~15; }
 
 // n cut into equal tiles of at most `most`, a tile a multiple of `unit`
 inline int tile_of(int64_t n, int most, int unit) {
+  if (n <= most) return int(std::min<int64_t>(most, (n + unit - 1) / unit * unit));
   const int64_t t = (n + most - 1) / most;
   const int64_t w = (n + t - 1) / t;
   return int(std::min<int64_t>(most, (w + unit - 1) / unit * unit));
@@ -90,9 +91,63 @@ bool f64_run_plain(int forms, bool small, bool plain) {
   return plain || small;
 }
 
+namespace {
+
+// the plain form alone: every problem by itself, rows of A as rows; one pass
+void build_plain(F64PlanHost& out, const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s) {
+  out.rowref.resize(s.size());
+  out.colref.resize(s.size());
+  out.rows.resize(p.size());
+  out.tiles.resize(p.size());
+  out.pieces.resize(p.size() + 1);
+  F64Ref *ra = out.rowref.data(), *rb = out.colref.data();
+  F64Row* row = out.rows.data();
+  F64Unit* tile = out.tiles.data();
+  int* piece = out.pieces.data();
+  int ns = 0, nt = 0, np = 0;
+  bool any_long = false;
+  for (const GemmProb& q : p) {
+    if (q.M <= 0 || q.N <= 0) continue;
+    const int cs = ns;
+    int noct = 0;
+    for (const GemmSeg *g = s.data() + q.s0, *e = s.data() + q.s1; g < e; ++g) {
+      if (g->K <= 0) continue;
+      ra[ns] = F64Ref{g->A, g->lda, 2 * g->K + (g->ta ? 1 : 0)};
+      rb[ns] = F64Ref{g->B, g->ldb, 2 * g->K + (g->tb ? 0 : 1)};
+      ++ns;
+      noct += int(unsigned(g->K + 7) >> 3);
+    }
+    any_long = any_long || noct >= F64_LONG;
+    row[nt] = F64Row{q.C, q.alpha, q.ldc, cs, 0, 2 * q.M + (q.accumulate ? 1 : 0)};
+    tile[nt] = F64Unit{nt, 1, 0, q.M, 0, q.N, cs, ns - cs, 0, 0, noct, 0, -1};
+    piece[nt] = np;
+    np += int((unsigned(q.M) + F64_PR - 1) / F64_PR * ((unsigned(q.N) + F64_PC - 1) / F64_PC));
+    ++nt;
+  }
+  piece[nt] = np;
+  out.rowref.resize(size_t(ns));
+  out.colref.resize(size_t(ns));
+  out.rows.resize(size_t(nt));
+  out.tiles.resize(size_t(nt));
+  out.pieces.resize(nt ? size_t(nt) + 1 : 0);
+  if (any_long) order_tiles(out);
+}
+
+}  // namespace
+
 F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int nsm, int what) {
-  const bool want_units = what & F64_UNITS, want_tiles = what & F64_TILES;
   F64PlanHost out;
+  f64_build_plan(out, p, s, nsm, what);
+  return out;
+}
+
+void f64_build_plan(F64PlanHost& out, const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int nsm, int what) {
+  out.clear();
+  if (!(what & F64_UNITS)) {
+    build_plain(out, p, s);
+    return;
+  }
+  const bool want_tiles = what & F64_TILES;
   const int np = int(p.size());
   // segments with K > 0, per problem (the caller's list itself when it holds nothing else)
   std::vector<int> f0(size_t(np) + 1, 0);
@@ -125,36 +180,7 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     whole = false;
   }
   const std::vector<GemmSeg>& seg = whole ? s : kept;
-  if (use.empty()) return out;
-
-  // the plain form alone: every problem by itself, rows of A as rows
-  if (!want_units) {
-    out.rowref.resize(seg.size());
-    out.colref.resize(seg.size());
-    for (size_t k = 0; k < seg.size(); ++k) {
-      const GemmSeg& g = seg[k];
-      out.rowref[k] = F64Ref{g.A, g.lda, 2 * g.K + (g.ta ? 1 : 0)};
-      out.colref[k] = F64Ref{g.B, g.ldb, 2 * g.K + (g.tb ? 0 : 1)};
-    }
-    out.rows.reserve(use.size());
-    out.tiles.reserve(use.size());
-    for (int i : use) {
-      const GemmProb& q = p[size_t(i)];
-      F64Unit u{};
-      u.cs = f0[size_t(i)];
-      u.nseg = f0[size_t(i) + 1] - u.cs;
-      for (int k = u.cs; k < u.cs + u.nseg; ++k) u.noct += (seg[size_t(k)].K + 7) / 8;
-      u.pos0 = int(out.rows.size());
-      u.npos = 1;
-      u.part = -1;
-      out.rows.push_back(F64Row{q.C, q.alpha, q.ldc, u.cs, 0, 2 * q.M + (q.accumulate ? 1 : 0)});
-      u.rows = q.M;
-      u.nt = q.N;
-      out.tiles.push_back(u);
-    }
-    order_tiles(out);
-    return out;
-  }
+  if (use.empty()) return;
 
   // 1. lists shared on the B side (rows stacked) and on the A side (columns stacked)
   auto same_b = [&](int i, int j) {
@@ -385,7 +411,6 @@ F64PlanHost f64_build_plan(const std::vector<GemmProb>& p, const std::vector<Gem
     for (size_t i = 0; i < units.size(); ++i) out.units[at[size_t(top - keys[i])]++] = units[i];
   }
   if (want_tiles) order_tiles(out);
-  return out;
 }
 
 }  // namespace dmrg

@@ -870,8 +870,9 @@ class CudaExec : public Exec {
 
   int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int forms) override {
     const bool small = f64_small(p, s);
-    const F64PlanHost h = f64_build_plan(
-        p, s, nsm_, (forms & GEMM_ANY && !small ? F64_UNITS : 0) | (forms & GEMM_PLAIN || small ? F64_TILES : 0));
+    F64PlanHost& h = lists_;
+    f64_build_plan(h, p, s, nsm_,
+                   (forms & GEMM_ANY && !small ? F64_UNITS : 0) | (forms & GEMM_PLAIN || small ? F64_TILES : 0));
     Plan pl;
     pl.forms = forms;
     pl.small = small;
@@ -916,6 +917,7 @@ class CudaExec : public Exec {
     pl.reds = reinterpret_cast<F64Red*>(d + off[4]);
     pl.tiles = reinterpret_cast<F64Unit*>(d + off[5]);
     pl.pieces = reinterpret_cast<int*>(d + off[6]);
+    if (h.capacity_bytes() > kListsMax) lists_ = F64PlanHost();
     pl.live = true;
     for (size_t i = 0; i < plans_.size(); ++i)
       if (!plans_[i].live) {
@@ -1436,12 +1438,14 @@ class CudaExec : public Exec {
   int64_t n_alloc_ = 0;
   cudaMemPool_t mpool_ = nullptr;
   static constexpr size_t kStageMax = size_t(512) << 20;   // pinned staging ring: at most 512 MiB
+  static constexpr size_t kListsMax = size_t(64) << 20;    // host lists kept between plans
   char* stage_ = nullptr;
   size_t stage_cap_ = 0, stage_head_ = 0;
   cudaEvent_t stage_ev_ = nullptr;
   std::vector<cudaGraphExec_t> graphs_;
   double* part_ = nullptr;
   std::vector<Plan> plans_;
+  F64PlanHost lists_;   // host lists of the last plan, kept for the next one's
   std::weak_ptr<double> sums_;
   size_t sums_n_ = 0;
 };

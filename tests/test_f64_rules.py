@@ -69,3 +69,8 @@ ANY, PLAIN = 1, 2
     (ANY | PLAIN, 1, 0, 1), (ANY, 0, 1, -1), (ANY, 1, 1, -1), (PLAIN, 0, 0, -1), (PLAIN, 1, 0, -1), (0, 0, 0, -1)])
 def test_a_plan_runs_only_in_a_form_it_was_built_for(lib, forms, small, plain, route):
     assert lib.f64_route(forms, small, plain) == route
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_lists_of_an_earlier_plan_leave_nothing(lib, seed):
+    assert lib.f64_reused_lists(seed) == 0
