@@ -64,10 +64,12 @@ typedef enum {
 
 /* precision of the sigma GEMMs.  FP64 products of some size run on the tensor cores, as
  * exact products of 8-bit digits: 62 bits of a row's (column's) largest element over up
- * to 192 k.  Their error is that of FP64 normwise; an element of a result whose terms are
- * all far below its row's largest element times its column's is within 2^-36 of the sum of
- * their magnitudes.  dmrg_davidson of an FP64 handle and the operators of a loaded basis
- * use FP64 multiply-adds throughout. */
+ * to 192 k.  Normwise their error is that of FP64 multiply-adds.  In the calls that return
+ * sigma, densities or an expectation value, an element whose terms are all far below its
+ * row's largest element times its column's is also within 2^-36 of the sum of their
+ * magnitudes; the iterations and truncations of sweeps, the FP64 refinement of split-BF16
+ * solves and dmrg_eigh_batch's eigenvectors have the normwise bound alone.  dmrg_davidson
+ * of an FP64 handle and the operators of a loaded basis use multiply-adds throughout. */
 enum {
   DMRG_PREC_FP64 = 0,        /* FP64 operands, FP64 accumulation */
   DMRG_PREC_MIXED_BF16 = 1   /* split BF16 operands on tcgen05, FP32 accumulation */

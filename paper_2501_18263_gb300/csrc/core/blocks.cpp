@@ -873,8 +873,8 @@ void Engine::renormalize(bool left, const Enlarged& E, const OpSet& eops, const 
   std::vector<GemmSeg> s1, s2;
   int64_t used = 0;
   auto flush = [&]() {
-    if (!p1.empty()) ex_->gemm(p1, s1, plain);
-    if (!p2.empty()) ex_->gemm(p2, s2, plain);
+    if (!p1.empty()) ex_->gemm(p1, s1, plain ? Fp64::plain : Fp64::norm);
+    if (!p2.empty()) ex_->gemm(p2, s2, plain ? Fp64::plain : Fp64::norm);
     p1.clear(); p2.clear(); s1.clear(); s2.clear();
     used = 0;
   };

@@ -252,9 +252,11 @@ class Engine {
   int64_t psi_size() const { return psi_n_; }
   const BondStats& stats() const { return st_; }
 
-  void sigma(const double* psi, double* sig, bool plain = false);   // device pointers, FP64 path
-  void sigma_body(int precision);   // kernels of one sigma, psi_in_ -> sig_out_ (kPlain: FP64 multiply-adds)
-  static constexpr int kPlain = 2;
+  void sigma(const double* psi, double* sig, Fp64 how = Fp64::fine);   // device pointers, FP64 path
+  // kernels of one sigma, psi_in_ -> sig_out_, at a DMRG_PREC_* (FP64: fine) or in one of
+  // the other forms of FP64 products
+  void sigma_body(int precision);
+  static constexpr int kMixed = 1, kPlain = 2, kNorm = 3;
   // the same, from the bond's captured graph when possible (captured on first use
   // unless allow_capture is false: capturing instantiates a graph)
   void sigma_run(int precision, bool allow_capture = true);
@@ -404,9 +406,9 @@ class Engine {
   int mplan_hl_ = -1;
   float* part_ = nullptr;
   int nparts_ = 1;
-  // one captured CUDA graph per prepared bond and precision for the sigma steps of
+  // one captured CUDA graph per prepared bond and form of sigma for the sigma steps of
   // Davidson (psi copied into psi_in_, result read from sig_out_ around the replay)
-  int graph_[3] = {-1, -1, -1};
+  int graph_[4] = {-1, -1, -1, -1};
   int64_t graph_runs_ = 0;
   void free_mixed();
   // sweep state

@@ -184,7 +184,7 @@ double Engine::davidson(double* psi, double tol, int max_iter, int max_sub, int*
   const int prec = P_.precision;
 
   auto apply = [&](const double* in, double* out, int pr) {
-    if (pr == 0) sigma(in, out, plain);
+    if (pr == 0) sigma(in, out, plain ? Fp64::plain : Fp64::norm);
     else sigma_precision(in, out, pr);
   };
 
@@ -450,7 +450,7 @@ void Engine::truncate_and_move(bool ltr, int D, double* trunc_w, std::vector<int
       q.s1 = int(S.size());
       P.push_back(q);
     }
-    ex_->gemm(P, S);
+    ex_->gemm(P, S, Fp64::norm);
   }
   {
     std::vector<double*> Av, wvv, Zv;
@@ -565,7 +565,7 @@ void Engine::truncate_and_move(bool ltr, int D, double* trunc_w, std::vector<int
       q.s1 = int(S.size());
       P.push_back(q);
     }
-    ex_->gemm(P, S);
+    ex_->gemm(P, S, Fp64::norm);
   }
   // renormalise the operators of the enlarged block that was truncated
   Enlarged Eold = E;
@@ -653,7 +653,7 @@ void Engine::truncate_and_move(bool ltr, int D, double* trunc_w, std::vector<int
           P.push_back(q);
         }
     }
-    ex_->gemm(P, S);
+    ex_->gemm(P, S, Fp64::norm);
   }
   ex_->release(Y);
   if (psi_cur_) ex_->release(psi_cur_);

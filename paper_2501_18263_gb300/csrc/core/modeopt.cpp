@@ -176,7 +176,7 @@ std::vector<double> Engine::left_spectrum(const double* psi) {
     q.s1 = int(S.size());
     P.push_back(q);
   }
-  ex_->gemm(P, S);
+  ex_->gemm(P, S, Fp64::norm);
   std::vector<double*> Av, wvv, Zv;
   int64_t wo = 0;
   for (size_t k = 0; k < blk.size(); ++k) {

@@ -965,7 +965,7 @@ void Engine::build_sigma_plan() {
     }
     ex_->diag(diag_tasks_);
     diag_plan_ = ex_->gemm_plan(PD, SD, GEMM_PLAIN);
-    ex_->gemm_run(diag_plan_, true);
+    ex_->gemm_run(diag_plan_, Fp64::plain);
   }
 }
 
@@ -973,13 +973,13 @@ void Engine::build_sigma_plan() {
 // replayed from a captured CUDA graph (one per bond and precision) when the
 // stream allows it, otherwise issued directly.
 void Engine::sigma_body(int precision) {
-  const bool plain = precision == kPlain;
-  if (precision == 0 || plain || !mixed_ready_) {
+  if (precision != kMixed || !mixed_ready_) {
+    const Fp64 how = precision == kPlain ? Fp64::plain : precision == kNorm ? Fp64::norm : Fp64::fine;
     for (auto& c : chunks_) {
-      if (c.plan1 >= 0) ex_->gemm_run(c.plan1, plain);
-      ex_->gemm_run(c.plan2, plain);
+      if (c.plan1 >= 0) ex_->gemm_run(c.plan1, how);
+      ex_->gemm_run(c.plan2, how);
     }
-    if (plan_hl_ >= 0) ex_->gemm_run(plan_hl_, plain);
+    if (plan_hl_ >= 0) ex_->gemm_run(plan_hl_, how);
     return;
   }
   ex_->split_run(psi_split_);
@@ -995,7 +995,7 @@ void Engine::sigma_body(int precision) {
 }
 
 void Engine::sigma_run(int precision, bool allow_capture) {
-  const int k = precision == kPlain ? 2 : (precision == 0 || !mixed_ready_) ? 0 : 1;
+  const int k = precision == kMixed && !mixed_ready_ ? 0 : precision;
   if (allow_capture && graph_[k] < 0 && !ex_->profiling())
     graph_[k] = ex_->graph_capture([&] { sigma_body(precision); });
   if (graph_[k] >= 0 && !ex_->profiling()) {
@@ -1006,10 +1006,10 @@ void Engine::sigma_run(int precision, bool allow_capture) {
   }
 }
 
-void Engine::sigma(const double* psi, double* sig, bool plain) {
+void Engine::sigma(const double* psi, double* sig, Fp64 how) {
   if (bond_ < 0) throw std::runtime_error("sigma: no bond prepared");
   ex_->d2d(psi_in_, psi, psi_n_ * sizeof(double));
-  sigma_run(plain ? kPlain : 0);
+  sigma_run(how == Fp64::plain ? kPlain : how == Fp64::norm ? kNorm : 0);
   ex_->d2d(sig, sig_out_, psi_n_ * sizeof(double));
 }
 

@@ -122,6 +122,22 @@ struct SplitTask {
 
 enum { GEMM_ANY = 1, GEMM_PLAIN = 2 };
 
+// How an FP64 product may be formed.
+//  fine   FP64 multiply-adds or exact digit products on the tensor cores: every element of
+//         a chunk's sum within 2^-36 of the sum of its terms' magnitudes (f64_digits.h;
+//         multiply-adds: k 2^-53), and normwise as multiply-adds
+//  norm   the same without the first: errors of the size of FP64 rounding relative to the
+//         row's largest element times the column's, so that an element whose terms are all
+//         far below that loses bits.  For steps whose results are used, and limited by
+//         other errors, as vectors or matrices: a sweep's iterations and truncations, and
+//         the eigensolver's products of orthogonal matrices
+//  plain  multiply-adds in the order of the segments and k: rounding that does not depend
+//         on the launch
+// A real state makes the difference in cost: half the elements of X = O psi can be zero by
+// spin symmetry, up to noise, and fine forms each of them again (two sweeps at L = 16,
+// D = 256: FP64 products 1.13 s, 2.82 s with fine)
+enum class Fp64 { fine, norm, plain };
+
 class Exec {
  public:
   virtual ~Exec() {}
@@ -145,17 +161,12 @@ class Exec {
 
   // grouped element-wise Kronecker accumulation (operator blocking)
   virtual void kron(const std::vector<KronGroup>& g, const std::vector<KronTask>& t) = 0;
-  // grouped, segmented FP64 GEMM (one-shot upload).  plain: every element by FP64
-  // multiply-adds in the order of its segments and k, so that its rounding does not
-  // depend on the launch; otherwise the executor may use its tensor-core form: another
-  // rounding sequence, errors of the size of FP64 rounding relative to the row's largest
-  // element times the column's (normwise no larger), and within 2^-36 of every element's
-  // own terms (f64_digits.h), where multiply-adds are within k 2^-53
-  virtual void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain = false) = 0;
+  // grouped, segmented FP64 GEMM (one-shot upload)
+  virtual void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, Fp64 how = Fp64::fine) = 0;
   // persistent plans (uploaded once, replayed during Davidson); forms: what gemm_run may
-  // be asked for (GEMM_ANY: plain = false, GEMM_PLAIN: plain = true, or both)
+  // be asked for (GEMM_ANY: fine and norm, GEMM_PLAIN: plain, or both)
   virtual int gemm_plan(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, int forms) = 0;
-  virtual void gemm_run(int plan, bool plain = false) = 0;
+  virtual void gemm_run(int plan, Fp64 how = Fp64::fine) = 0;
   virtual void plan_free(int plan) = 0;
   virtual void diag(const std::vector<DiagTask>& t) = 0;
   // generalised Fock matrix F_pq = sum_r t_pr g1_qr + sum_rst v_prst g2_qrst and the

@@ -927,9 +927,9 @@ class CudaExec : public Exec {
     plans_.push_back(pl);
     return int(plans_.size() - 1);
   }
-  void gemm_run(int id, bool plain) override {
+  void gemm_run(int id, Fp64 how) override {
     Plan& pl = plans_.at(id);
-    plain = f64_run_plain(pl.forms, pl.small, plain);
+    const bool plain = f64_run_plain(pl.forms, pl.small, how == Fp64::plain);
     if (!(plain ? pl.ntiles : pl.nunits)) return;   // no outputs
     launch(PROF_GEMM, [&] {
       if (plain) {
@@ -938,7 +938,7 @@ class CudaExec : public Exec {
         return;
       }
       launch_gemm_f64_tc(pl.units, pl.nunits, pl.rows, pl.rowref, pl.colref, pl.part.get(), pl.reds, pl.nreds, pl.next, err_, nsm_,
-                         st_);
+                         how == Fp64::fine, st_);
     });
   }
   void free_plan_mem(Plan& p) {
@@ -948,10 +948,10 @@ class CudaExec : public Exec {
     p.live = false;
   }
   void plan_free(int id) override { free_plan_mem(plans_.at(id)); }
-  void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, bool plain) override {
+  void gemm(const std::vector<GemmProb>& p, const std::vector<GemmSeg>& s, Fp64 how) override {
     if (p.empty()) return;
-    int id = gemm_plan(p, s, plain ? GEMM_PLAIN : GEMM_ANY);
-    gemm_run(id, plain);
+    int id = gemm_plan(p, s, how == Fp64::plain ? GEMM_PLAIN : GEMM_ANY);
+    gemm_run(id, how);
     plan_free(id);
   }
   void orbital_gradient(int L, const double* t, const double* v, const double* g1, const double* g2,
@@ -1416,7 +1416,7 @@ class CudaExec : public Exec {
         q.s1 = int(S.size());
         P.push_back(q);
       }
-      gemm(P, S, false);
+      gemm(P, S, Fp64::norm);
     }
     // 5. order
     launch(PROF_EIG, [&] { syev_sort_kernel<<<unsigned((ncol + 255) / 256), 256, 0, st_>>>(dj, dpn, nj); });

@@ -14,8 +14,8 @@
 // accumulators are combined in integers, rounded once to FP64 and added over the chunks
 // in FP64.  The error is normwise: an element 2^9 or more below its row's largest is held
 // in fewer than 53 bits.  Elements of C whose chunk sum comes out far below what its row
-// and column could give (f64_weak), and rows or columns with an infinity or a NaN, are
-// computed by plain FP64 multiply-adds.
+// and column could give (f64_weak; FINE only), and rows or columns with an infinity or a
+// NaN, are computed by plain FP64 multiply-adds.
 //
 // One tile: 128 rows (TMEM lanes) x up to 64 columns, eight accumulators of 64 TMEM
 // columns.  With B's digits stored one after the other along N, one MMA of digit i of
@@ -270,6 +270,7 @@ __device__ __forceinline__ void store_digits(double x0, double x1, int e, uint32
   }
 }
 
+template <bool FINE>
 __global__ void __maxnreg__(REGS)
     gemm_f64_tc_kernel(const F64Unit* __restrict__ units, int nunits, const F64Row* __restrict__ rows,
                        const F64Ref* __restrict__ rowref, const F64Ref* __restrict__ colref,
@@ -702,7 +703,7 @@ __global__ void __maxnreg__(REGS)
               v[i] = f64_assemble_fast(hi, lo, ea, max(S.expo[F64_TM + min(cb + hh + i, nt - 1)] >> 20, 1), flip, &bd,
                                        &lead);
               bad |= bd && rv;
-              again |= f64_weak(lead) ? 1u << i : 0u;
+              if (FINE && f64_weak(lead)) again |= 1u << i;
             }
             if (__any_sync(0xffffffffu, bad)) {   // results outside the normal range
 #pragma unroll
@@ -713,7 +714,7 @@ __global__ void __maxnreg__(REGS)
                 v[i] = assemble_any(hi, lo, ea, max(S.expo[F64_TM + min(cb + hh + i, nt - 1)] >> 20, 1), flip);
               }
             }
-            if (special || __any_sync(0xffffffffu, again != 0)) {
+            if (special || (FINE && __any_sync(0xffffffffu, again != 0))) {
               const int xa = rv ? S.expo[r] : 0;
 #pragma unroll
               for (int i = 0; i < 4; ++i) {   // (a sum of nothing but zeros is one)
@@ -826,10 +827,11 @@ __global__ void __launch_bounds__(256) gemm_f64_reduce_kernel(const F64Red* __re
 
 }  // namespace
 
-void launch_gemm_f64_tc(const F64Unit* units, int nunits, const F64Row* rows, const F64Ref* rowref,
-                        const F64Ref* colref, double* part, const F64Red* reds, int nreds, int* next, int* err, int nsm,
-                        cudaStream_t st) {
-  if (nunits <= 0) return;
+namespace {
+
+template <bool FINE>
+void launch_tc(const F64Unit* units, int nunits, const F64Row* rows, const F64Ref* rowref, const F64Ref* colref,
+               double* part, int* next, int* err, int nsm, cudaStream_t st) {
   // the shared-memory opt-in is a per-device attribute of the kernel (devices past 63
   // set it on every launch)
   static std::atomic<uint64_t> attr_set{0};
@@ -839,14 +841,24 @@ void launch_gemm_f64_tc(const F64Unit* units, int nunits, const F64Row* rows, co
   if (!bit || !(attr_set.load(std::memory_order_relaxed) & bit)) {
     // the register split in the kernel draws on exactly REGS registers per thread
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, gemm_f64_tc_kernel) != cudaSuccess || fa.numRegs != REGS)
+    if (cudaFuncGetAttributes(&fa, gemm_f64_tc_kernel<FINE>) != cudaSuccess || fa.numRegs != REGS)
       throw CudaError("gemm_f64_tc_kernel: built with another register count");
-    if (cudaFuncSetAttribute(gemm_f64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) ==
+    if (cudaFuncSetAttribute(gemm_f64_tc_kernel<FINE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) ==
         cudaSuccess)
       attr_set.fetch_or(bit, std::memory_order_relaxed);
   }
   const int grid = nunits < nsm ? nunits : nsm;
-  gemm_f64_tc_kernel<<<grid, THREADS, SMEM_BYTES, st>>>(units, nunits, rows, rowref, colref, part, next, err);
+  gemm_f64_tc_kernel<FINE><<<grid, THREADS, SMEM_BYTES, st>>>(units, nunits, rows, rowref, colref, part, next, err);
+}
+
+}  // namespace
+
+void launch_gemm_f64_tc(const F64Unit* units, int nunits, const F64Row* rows, const F64Ref* rowref,
+                        const F64Ref* colref, double* part, const F64Red* reds, int nreds, int* next, int* err, int nsm,
+                        bool fine, cudaStream_t st) {
+  if (nunits <= 0) return;
+  if (fine) launch_tc<true>(units, nunits, rows, rowref, colref, part, next, err, nsm, st);
+  else launch_tc<false>(units, nunits, rows, rowref, colref, part, next, err, nsm, st);
   if (nreds > 0) gemm_f64_reduce_kernel<<<dim3(unsigned(nreds), 4), 256, 0, st>>>(reds, rows, part);
 }
 

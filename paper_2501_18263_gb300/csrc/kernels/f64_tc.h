@@ -8,11 +8,12 @@ namespace dmrg {
 
 // one launch over the units of a plan and, when some are split over K, one over its
 // reductions; err is a device int that receives a nonzero code when a bounded wait
-// gives up; next: two device ints of the plan, zero before its first launch, through
+// gives up; fine: sums too small for their digits are computed again by multiply-adds
+// (f64_weak); next: two device ints of the plan, zero before its first launch, through
 // which the CTAs claim units (zero again when the launch ends)
 void launch_gemm_f64_tc(const F64Unit* units, int nunits, const F64Row* rows, const F64Ref* rowref,
                         const F64Ref* colref, double* part, const F64Red* reds, int nreds, int* next, int* err, int nsm,
-                        cudaStream_t st);
+                        bool fine, cudaStream_t st);
 
 // the same problems by plain FP64 multiply-adds, every element's terms in the order of
 // its segments and k: tiles (the first nlong, with plong pieces, are long sums) and the
