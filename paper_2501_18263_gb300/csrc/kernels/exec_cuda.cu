@@ -1276,8 +1276,9 @@ class CudaExec : public Exec {
     }
     // 1. the reduction: a cluster of SYEV_CLUSTER CTAs for each matrix of order >= 64
     // (largest first), one CTA for each smaller one, whose arithmetic one SM does in the
-    // time a cluster takes for its barriers (the batch of syev_tridiag_kernel: 8.6 ms in
-    // all with the line at 48 or 64, 8.8 at 80, 9.2 at 112, 9.8 at 160); 2. Q
+    // time a cluster takes for its barriers (the batch of syev_tridiag_kernel, with its
+    // faster update and leaves: 8.6 ms in all with the line at 48 or 64, 8.8 at 80, 9.2 at
+    // 112, 9.8 at 160); 2. Q
     std::vector<int> small, big;
     for (int j = 0; j < nj; ++j) (n[j] >= 64 ? big : small).push_back(j);
     std::stable_sort(big.begin(), big.end(), [&](int a, int b) { return n[size_t(a)] > n[size_t(b)]; });

@@ -87,7 +87,7 @@ F64_HD int f64_rint(float x) {
 // The product sum of a chunk: a[w] = sum_k sum_{i + j = w} da_i db_j (exact integers for
 // w < 6; |a[0]| < 2^20, |a[1]| < 2^22, |a[2]| < 2^23, the others below 2^25), so
 // sum_k Xa Xb = 2^56 (V + what the weights above 7 hold) with V = sum_w a[w] 2^(8 (7 - w)),
-// given as hi 2^32 + lo (weight 7 rounded into weight 6: 2^-62 of the largest product).
+// given as hi 2^32 + lo (weight 7 rounded into weight 6: 2^-60 of the largest product).
 // Shifts and adds only: a 64-bit integer multiply-add runs on the slow FP64 pipe.
 F64_HD void f64_combine(float a0, float a1, float a2, float a3, float a4, float a5, float a6, float a7, int64_t& hi,
                         uint32_t& lo) {
